@@ -275,7 +275,7 @@ extern "C" vd_status vd_create(const vd_window_desc* desc, const vd_params* para
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        sms <= 0 || vd_pose_prepare() != cudaSuccess) {
+        sms <= 0 || vd_pose_prepare() != cudaSuccess || vd_depth_prepare() != cudaSuccess) {
       vd_set_error("cannot query the device");
       delete c;
       return VD_ERR_CUDA;

@@ -2,6 +2,10 @@
 // and argmin (parallel phase) followed by propagation along alternately
 // directed 1-D chains (sequential phase), plus the hierarchical option
 // (coarse global pass + local full-resolution windows).
+#include <limits.h>
+
+#include <algorithm>
+
 #include "vd_device.cuh"
 
 #define VD_DISPATCH_NF(N, KERNEL_CALL)      \
@@ -401,195 +405,153 @@ VD_UNROLL(VD_KQ_PRE_UNROLL)
 // rho_new = rho* unless the predecessor's new value has strictly lower
 // energy; `restart` > 0 starts afresh every `restart` pixels (local windows
 // of the hierarchical scheme).
+//
+// A block takes one chain and keeps, per pixel, its value x and the incoming
+// value `in` it was decided with, in shared memory.  First every pixel is
+// decided as if its predecessor kept its own rho* (all energies independent
+// of one another).  A pixel whose `in` is no longer its
+// predecessor's x is pending.  Each round gives every pending pixel an equal
+// share w of the threads and tries its incoming value v at the next w pixels
+// at once: up to the first pixel that rejects v, that already holds what it
+// would get, or that is pending itself, the sequential walk writes v; the
+// pixel after the last one written is the only one that can become pending.
+// So short corrections run side by side and a long run of one value is
+// followed blockDim.x pixels at a time.  Every round settles the first
+// pending pixel of a chain for good, and without a pending pixel every pixel
+// satisfies the definition: the result is exactly the sequential walk.
+// Bound: latency, about 4000 cycles from a pixel's loads to its decision,
+// times the rounds of the slowest chain (19 on a 1216 x 368 window with
+// N = 6, 4.5 on average; a run is 1.2 pixels long on average, the longest
+// 73).  A warp per chain, 38 pixels walked by each lane one after another,
+// took 125 us there and 98 us on 509 x 383 columns with N = 5; this takes 65
+// and 53.
 // ---------------------------------------------------------------------------
-// ---------------------------------------------------------------------------
-// K2, warp version: one warp per chain, lane i owns the contiguous segment
-// [i*seg, (i+1)*seg) of the chain.  Phase A: every lane walks its segment as
-// if its first pixel started the chain.  Correction rounds: a lane whose
-// incoming value (the predecessor lane's end value) changed walks again from
-// its segment start with that value and stops as soon as the carried value
-// equals what it wrote at that pixel before (the rest of the walk depends on
-// the carried value only, so it is unchanged).  The rounds end when no end
-// value changes, so the result is exactly the sequential walk.
-// ---------------------------------------------------------------------------
-// The loads of one pixel's propagation step that do not depend on the
-// carried value (its rigidness, X_1 at the pixel, the prior, rho* and E*),
-// issued one pixel ahead of the step that uses them, so that their latency
-// overlaps the current pixel's energy.
-template <int NF>
-struct VdPixLoads {
-  float q[NF];
-  float2 f1;
-  float pv, qh, pc;
-  float own, e;
-};
-
-template <int NF>
-__device__ __forceinline__ void vd_pix_load(VdPixLoads<NF>& L, const DevParams& P,
-                                            const float2* __restrict__ flow,
-                                            const float* __restrict__ q,
-                                            const float* __restrict__ prior_val,
-                                            const float* __restrict__ qhat,
-                                            const float* __restrict__ pconf,
-                                            const float* __restrict__ rho_star,
-                                            const float* __restrict__ e_star, size_t npix,
-                                            size_t j) {
-#pragma unroll
-  for (int t = 0; t < NF; ++t) L.q[t] = __ldg(q + (size_t)t * npix + j);
-  L.f1 = __ldg(flow + j);
-  L.pv = 0.0f;
-  L.qh = 0.0f;
-  L.pc = 0.0f;
-  if (P.prior_kind != VD_PRIOR_NONE) {
-    L.pv = __ldg(prior_val + j);
-    L.qh = __ldg(qhat + j);
-    L.pc = __ldg(pconf + j);
-  }
-  L.own = rho_star[j];
-  L.e = e_star[j];
+__device__ __forceinline__ bool vd_same_bits(float a, float b) {
+  return __float_as_uint(a) == __float_as_uint(b);
 }
 
-// vd_pixel_setup from the preloaded values (the same arithmetic).
-template <int NF>
-__device__ __forceinline__ void vd_pixel_from_loads(VdPixel<NF>& px, const DevParams& P,
-                                                    const float* __restrict__ sPose, int u, int v,
-                                                    const VdPixLoads<NF>& L) {
-  const float rx = ((float)u - P.cx) / P.fx;
-  const float ry = ((float)v - P.cy) / P.fy;
-#pragma unroll
-  for (int t = 0; t < NF; ++t) {
-    const float* M = sPose + 12 * (t + 1);
-    px.ax[t] = fmaf(M[0], rx, fmaf(M[1], ry, M[2]));
-    px.ay[t] = fmaf(M[3], rx, fmaf(M[4], ry, M[5]));
-    px.az[t] = fmaf(M[6], rx, fmaf(M[7], ry, M[8]));
-    px.wl[t] = L.q[t] * VD_LN2;
-  }
-  px.f1x = L.f1.x;
-  px.f1y = L.f1.y;
-  px.u = (float)u;
-  px.v = (float)v;
-  px.pw = 0.0f;
-  px.pv = 0.0f;
-  if (P.prior_kind != VD_PRIOR_NONE && isfinite(L.pv)) {
-    px.pv = L.pv;
-    px.pw = L.qh * L.pc;
-  }
-}
+#define VD_PROP_MAX_THREADS 256
+#define VD_PROP_ITEM_BYTES (2 * (int)sizeof(float) + 2 * (int)sizeof(unsigned short))
 
 template <int NF>
-__device__ __forceinline__ float vd_prop_step(const DevParams& P, const float* sPose,
-                                              const float2* __restrict__ flow,
-                                              const float* __restrict__ q,
-                                              const float* __restrict__ prior_val,
-                                              const float* __restrict__ qhat,
-                                              const float* __restrict__ pconf, float cur, float own,
-                                              float e_own, int u, int v, size_t j) {
-  const size_t npix = (size_t)P.W * P.H;
-  VdPixel<NF> px;
-  vd_pixel_setup<NF>(px, P, sPose, u, v, q, npix, j, flow, prior_val, qhat, pconf);
-  const float Ec = vd_energy_full<NF>(px, P, sPose, flow, npix, cur);
-  return (Ec < e_own) ? cur : own;
-}
-
-template <int NF>
-__global__ void __launch_bounds__(128)
-k_propagate_warp(DevParams P, const float* __restrict__ posef, const float2* __restrict__ flow,
-                 const float* __restrict__ q, const float* __restrict__ prior_val,
-                 const float* __restrict__ qhat, const float* __restrict__ pconf,
-                 const float* __restrict__ rho_star, const float* __restrict__ e_star,
-                 float* __restrict__ rho_new, int direction, int restart, int s) {
+__global__ void __launch_bounds__(VD_PROP_MAX_THREADS)
+k_propagate(DevParams P, const float* __restrict__ posef, const float2* __restrict__ flow,
+            const float* __restrict__ q, const float* __restrict__ prior_val,
+            const float* __restrict__ qhat, const float* __restrict__ pconf,
+            const float* __restrict__ rho_star, const float* __restrict__ e_star,
+            float* __restrict__ rho_new, int direction, int restart, int s) {
+  extern __shared__ float sX[];                 // x, then in, of every pixel, then two lists of pixels
   __shared__ float sPose[12 * (VD_MAX_FLOWS + 1)];
-  vd_load_pose_smem<NF>(sPose, posef);
+  __shared__ int sStop[VD_PROP_MAX_THREADS];    // 4 d + kind of the first pixel that ends a try
+  __shared__ int sCount[2];                     // pending pixels of this round and the next
   const bool rows = (direction & 1) == 0;
   const bool rev = direction >= 2;
   // s > 0: the chains of the coarse grid of representative pixels
   // (min(s uc, W - 1), min(s vc, H - 1)), written to the coarse map
   // rho_new[vc][uc] (the hierarchical scheme's global pass)
   const int Wc = s > 0 ? (P.W + s - 1) / s : P.W, Hc = s > 0 ? (P.H + s - 1) / s : P.H;
-  const int nchains = rows ? Hc : Wc;
   const int L = rows ? Wc : Hc;
-  const int ch = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (ch >= nchains) return;          // whole warps leave together
-  const int seg = (L + 31) >> 5;
-  const int m0 = min(L, lane * seg), m1 = min(L, m0 + seg);
-  // position m of the chain: pixel (u, v) and index j of the inputs, and the
-  // index of the output (j itself at full resolution)
-  auto pix = [&](int m, int* u, int* v, size_t* o) -> size_t {
-    const int pos = rev ? L - 1 - m : m;
+  const int ch = (int)blockIdx.x, T = (int)blockDim.x;
+  const size_t npix = (size_t)P.W * P.H;
+  float* sIn = sX + L;
+  unsigned short* sList = (unsigned short*)(sIn + L);
+  // position i of the chain: pixel (u, v) and index of the inputs, and the
+  // index of the output (the same at full resolution)
+  auto pix = [&](int i, int* u, int* v, size_t* o) -> size_t {
+    const int pos = rev ? L - 1 - i : i;
     const int uc = rows ? pos : ch, vc = rows ? ch : pos;
     *u = s > 0 ? min(uc * s, P.W - 1) : uc;
     *v = s > 0 ? min(vc * s, P.H - 1) : vc;
     *o = (size_t)vc * Wc + uc;
     return (size_t)VD_CHK(VD_SITE_CHAIN, (long long)(*v) * P.W + (*u), (long long)P.W * P.H);
   };
-  // phase A; the next pixel's loads are issued before this pixel's energy
-  const size_t npix = (size_t)P.W * P.H;
-  float cur = 0.0f;
-  VdPixLoads<NF> Ln;
-  int un = 0, vn = 0;
-  size_t jn = 0, on = 0;
-  if (m0 < m1) {
-    jn = pix(m0, &un, &vn, &on);
-    vd_pix_load<NF>(Ln, P, flow, q, prior_val, qhat, pconf, rho_star, e_star, npix, jn);
+  // the chain's first pixel and the first of every restart window take rho*
+  auto fresh = [&](int i) { return i == 0 || (restart > 0 && i % restart == 0); };
+  // value of pixel i under the incoming value c
+  auto decide = [&](int i, float c) {
+    int u, v;
+    size_t o;
+    const size_t j = pix(i, &u, &v, &o);
+    const float own = rho_star[j], e = e_star[j];
+    VdPixel<NF> px;
+    vd_pixel_setup<NF>(px, P, sPose, u, v, q, npix, j, flow, prior_val, qhat, pconf);
+    // every gathered flow's taps in flight at once: latency sets the pace
+    return vd_energy_full<NF>(px, P, sPose, flow, npix, c) < e ? c : own;
+  };
+  vd_load_pose_smem<NF>(sPose, posef);
+  for (int i = threadIdx.x; i < L; i += T) {
+    int u, v;
+    size_t o;
+    const float in = rho_star[pix(max(i - 1, 0), &u, &v, &o)];
+    sIn[i] = in;
+    sX[i] = fresh(i) ? rho_star[pix(i, &u, &v, &o)] : decide(i, in);
   }
-  for (int m = m0; m < m1; ++m) {
-    const VdPixLoads<NF> L = Ln;
-    const int u = un, v = vn;
-    const size_t o = on;
-    if (m + 1 < m1) {
-      jn = pix(m + 1, &un, &vn, &on);
-      vd_pix_load<NF>(Ln, P, flow, q, prior_val, qhat, pconf, rho_star, e_star, npix, jn);
-    }
-    if (m == m0 || (restart > 0 && m % restart == 0)) {
-      cur = L.own;
-    } else {
-      VdPixel<NF> px;
-      vd_pixel_from_loads<NF>(px, P, sPose, u, v, L);
-      // every gathered flow's taps in flight at once: the walk is a chain of
-      // dependent energies, so their latency, not their work, sets its pace
-      const float Ec = vd_energy_full<NF>(px, P, sPose, flow, npix, cur);
-      cur = (Ec < L.e) ? cur : L.own;
-    }
-    rho_new[o] = cur;
+  if (threadIdx.x < 2) sCount[threadIdx.x] = 0;
+  __syncthreads();
+  auto pending = [&](int i) { return !fresh(i) && !vd_same_bits(sX[i - 1], sIn[i]); };
+  // append i where p (whole warps call it together)
+  auto append = [&](unsigned short* list, int* count, int i, bool p) {
+    const int lane = threadIdx.x & 31;
+    const unsigned m = __ballot_sync(0xffffffffu, p);
+    int at = 0;
+    if (lane == 0 && m) at = atomicAdd(count, __popc(m));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+    if (p) list[at] = (unsigned short)i;
+  };
+  for (int b = 0; b < L; b += T) {
+    const int i = b + threadIdx.x;
+    append(sList, &sCount[0], i, i < L && pending(i));
   }
-  float end = cur;                     // value carried out of the segment
-  bool have_in = false;                // phase A assumed no incoming value
-  float last_in = 0.0f;
-  for (int round = 0; round < 32; ++round) {
-    float in = __shfl_up_sync(0xffffffffu, end, 1);
-    const bool has_pred = lane > 0 && m1 > m0 && m0 > 0;
-    bool walk = has_pred && (!have_in || in != last_in);
-    if (walk && restart > 0 && m0 % restart == 0) walk = false;   // forced fresh start
-    bool changed = false;
-    if (walk) {
-      have_in = true;
-      last_in = in;
-      float c = in;
-      bool merged = false;
-      for (int m = m0; m < m1; ++m) {
-        int u, v;
-        size_t o;
-        const size_t j = pix(m, &u, &v, &o);
-        const float own = rho_star[j];
-        float nc;
-        if (restart > 0 && m % restart == 0)
-          nc = own;
-        else
-          nc = vd_prop_step<NF>(P, sPose, flow, q, prior_val, qhat, pconf, c, own, e_star[j], u, v, j);
-        if (nc == rho_new[o]) {
-          merged = true;
-          break;
-        }
-        rho_new[o] = nc;
-        c = nc;
+  __syncthreads();
+  for (int r = 0; sCount[r] > 0; r ^= 1) {
+    const int total = sCount[r];
+    unsigned short* list = sList + (r ? L : 0);
+    unsigned short* next = sList + (r ? 0 : L);
+    for (int b = 0; b < total; b += T) {        // more than T: one pixel each
+      const int n = min(T, total - b), w = T / n;
+      const int f = (int)threadIdx.x / w, d = (int)threadIdx.x - f * w;
+      sStop[threadIdx.x] = INT_MAX;
+      int i = 0, kind = 3;                      // 3: nothing ends here
+      float v = 0.0f, x = 0.0f;
+      bool on = f < n;
+      if (on) {
+        const int i0 = list[b + f];
+        i = i0 + d;
+        v = sX[i0 - 1];
+        on = i < L && pending(i0);          // (a later part's may be settled by now)
+        if (on && d > 0 && pending(i)) kind = 2;   // pending itself: its own try
       }
-      if (!merged && c != end) {
-        end = c;
-        changed = true;
+      __syncthreads();                          // the state of this try is read
+      if (on && kind == 3) {
+        const bool fr = fresh(i);
+        x = fr ? sX[i] : decide(i, v);
+        if (vd_same_bits(x, sX[i])) kind = 0;   // holds it already: the rest stands
+        else if (!vd_same_bits(x, v)) kind = 1; // rejects v
       }
+      if (on && kind != 3) atomicMin(&sStop[f], 4 * d + kind);
+      __syncthreads();
+      const int stop = on ? sStop[f] : 0;
+      if (on && 4 * d <= stop && kind != 2) {
+        sX[i] = x;
+        sIn[i] = v;
+      }
+      __syncthreads();
+      // the pixel after the last one written may be pending now
+      // (after a merge the rest stands)
+      int after = L;
+      if (on && d == 0 && (stop == INT_MAX || (stop & 3) != 0))
+        after = i + (stop == INT_MAX ? w : (stop >> 2) + ((stop & 3) == 1 ? 1 : 0));
+      append(next, &sCount[r ^ 1], after, after < L && pending(after));
     }
-    if (!__any_sync(0xffffffffu, changed)) break;
+    __syncthreads();
+    if (threadIdx.x == 0) sCount[r] = 0;
+    __syncthreads();
+  }
+  for (int i = threadIdx.x; i < L; i += T) {
+    int u, v;
+    size_t o;
+    pix(i, &u, &v, &o);
+    rho_new[o] = sX[i];
   }
 }
 
@@ -675,20 +637,48 @@ cudaError_t launch_depth_sample(vd_ctx* c, uint32_t itcode, float s_pert, int nf
   return cudaGetLastError();
 }
 
+// Shared memory of the longest chain (16384 pixels), granted once per device
+// so that no launch, and no stream capture, has to change a function attribute.
+template <int NF>
+static cudaError_t prop_prepare() {
+  return cudaFuncSetAttribute(k_propagate<NF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              VD_PROP_ITEM_BYTES * 16384);
+}
+
+cudaError_t vd_depth_prepare(void) {
+  for (int n = 1; n <= VD_MAX_FLOWS; ++n) {
+    cudaError_t e = cudaSuccess;
+    VD_DISPATCH_NF(n, e = prop_prepare<NF>());
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// Threads of a block of k_propagate for a chain of L pixels: about ten
+// pixels a thread (measured with 1, 3, 6 and 10 on an earlier form of the
+// kernel: 1216-pixel rows 83, 81, 84 and 72 us, 383-pixel columns 72, 55, 58
+// and 57; more threads a chain leave fewer chains resident, and the later
+// rounds need few).
+static int prop_threads(int L) {
+  return std::min(VD_PROP_MAX_THREADS, std::max(64, (L / 10 + 31) / 32 * 32));
+}
+
+static size_t prop_smem(int L) { return (size_t)VD_PROP_ITEM_BYTES * L; }
+
 cudaError_t launch_depth_propagate(vd_ctx* c, int direction, int nf) {
   const bool rows = (direction & 1) == 0;
+  const int nch = rows ? c->H : c->W, L = rows ? c->W : c->H;
   if (!c->prm.hierarchical) {
-    const int nch = rows ? c->H : c->W;
-    VD_DISPATCH_NF(nf, (k_propagate_warp<NF><<<(nch + 3) / 4, 128, 0, c->stream>>>(
+    VD_DISPATCH_NF(nf, (k_propagate<NF><<<nch, prop_threads(L), prop_smem(L), c->stream>>>(
                               c->dp, c->posef, c->flow, c->q, c->prior_val, c->qhat, c->prior_conf,
                               c->rho_star, c->e_star, c->rho, direction, 0, 0)));
     return cudaGetLastError();
   }
   const int s = c->prm.hier_scale;
   const int Wc = (c->W + s - 1) / s, Hc = (c->H + s - 1) / s;
-  const int nchc = rows ? Hc : Wc;
   // global pass on the coarse grid: the same segmented exact chain walk
-  VD_DISPATCH_NF(nf, (k_propagate_warp<NF><<<(nchc + 3) / 4, 128, 0, c->stream>>>(
+  const int Lc = rows ? Wc : Hc;
+  VD_DISPATCH_NF(nf, (k_propagate<NF><<<rows ? Hc : Wc, prop_threads(Lc), prop_smem(Lc), c->stream>>>(
                             c->dp, c->posef, c->flow, c->q, c->prior_val, c->qhat, c->prior_conf,
                             c->rho_star, c->e_star, c->coarse, direction, 0, s)));
   cudaError_t e = cudaGetLastError();
@@ -700,8 +690,7 @@ cudaError_t launch_depth_propagate(vd_ctx* c, int direction, int nf) {
                             c->rho_star, c->e_star, c->coarse, s, c->rho_mid, c->e_mid)));
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int nch = rows ? c->H : c->W;
-  VD_DISPATCH_NF(nf, (k_propagate_warp<NF><<<(nch + 3) / 4, 128, 0, c->stream>>>(
+  VD_DISPATCH_NF(nf, (k_propagate<NF><<<nch, prop_threads(L), prop_smem(L), c->stream>>>(
                             c->dp, c->posef, c->flow, c->q, c->prior_val, c->qhat, c->prior_conf,
                             c->rho_mid, c->e_mid, c->rho, direction, c->prm.hier_window, 0)));
   return cudaGetLastError();

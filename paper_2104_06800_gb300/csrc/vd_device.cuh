@@ -152,8 +152,13 @@ __device__ __forceinline__ float vd_l2_beta2(const DevParams& P, float r2) {
   // beta = 2: P0 / p1 = P0 pi alpha^2 (1 + r^2 / alpha^2)^2
   const float s = fmaf(r2, P.inv_a2, 1.0f);
   const float y = P.c0 * s * s;
-  if (y < 1e30f) return vd_ell2(y);
-  return fmaf(2.0f, __log2f(s), P.log2c0);
+  // one logarithm and no branch: of 1 + y, or of s where y would overflow
+  const bool mid = y < 1e30f;
+  const float L = __log2f(mid ? 1.0f + y : s);
+  const float ser =
+      y * fmaf(y, fmaf(y, fmaf(y, fmaf(y, 0.2f, -0.25f), 0.33333334f), -0.5f), 1.0f) *
+      1.44269504f;
+  return y < 0.03125f ? ser : (mid ? L : fmaf(2.0f, L, P.log2c0));
 }
 
 // The flow term's log2(1 + P0 / p1): alpha = alpha0 + alpha1 |X_t(x)|.
@@ -312,30 +317,46 @@ __device__ __forceinline__ float vd_energy_full(const VdPixel<NF>& px, const Dev
     xs[t] = hx * iz;
     ys[t] = hy * iz;
   }
-  float2 F[NF];
+  // flow t is read at the pixel's position in frame t; every position is
+  // bounded first and every tap loaded without a branch (a branch per flow
+  // would wait for its loads before it issues the next flow's)
+  float2 f00[NF], f01[NF], f10[NF], f11[NF];
+  float wx[NF], wy[NF];
   bool ob[NF];
-  F[0] = make_float2(px.f1x, px.f1y);
   ob[0] = true;
 #pragma unroll
-  for (int t = 1; t < NF; ++t) {   // flow t read at the pixel's position in frame t
+  for (int t = 1; t < NF; ++t) {
     ob[t] = fr[t - 1] && vd_inside(xs[t - 1], ys[t - 1], P.W, P.H);
-    F[t] = make_float2(0.0f, 0.0f);
-    if (ob[t]) F[t] = vd_bilinear(flow + (size_t)t * npix, P.W, P.H, xs[t - 1], ys[t - 1]);
+    const float x = ob[t] ? xs[t - 1] : 0.0f, y = ob[t] ? ys[t - 1] : 0.0f;
+    const int x0 = min(__float2int_rd(x), P.W - 2);
+    const int y0 = min(__float2int_rd(y), P.H - 2);
+    wx[t] = x - (float)x0;
+    wy[t] = y - (float)y0;
+    const float2* p = flow + (size_t)t * npix +
+                      VD_CHK(VD_SITE_BILINEAR, (long long)y0 * P.W + x0,
+                             (long long)P.W * P.H - P.W - 1);
+    f00[t] = __ldg(p);
+    f01[t] = __ldg(p + 1);
+    f10[t] = __ldg(p + P.W);
+    f11[t] = __ldg(p + P.W + 1);
   }
   float E = vd_prior_energy<NF>(px, P, c);
 #pragma unroll
   for (int t = 0; t < NF; ++t) {
     const float xp = t == 0 ? px.u : xs[t - 1], yp = t == 0 ? px.v : ys[t - 1];
-    float l2;
-    if (ob[t] && fr[t]) {
-      const float dx = F[t].x - (xs[t] - xp);
-      const float dy = F[t].y - (ys[t] - yp);
-      const float r2 = fmaf(dx, dx, dy * dy);
-      l2 = vd_l2_flow(P, r2, fmaf(F[t].x, F[t].x, F[t].y * F[t].y));
-    } else {
-      l2 = ob[t] ? (VD_L_BEHIND / VD_LN2) : 0.0f;
+    float2 F = make_float2(px.f1x, px.f1y);
+    if (t > 0) {
+      const float tx = fmaf(wx[t], f01[t].x - f00[t].x, f00[t].x);
+      const float ty = fmaf(wx[t], f01[t].y - f00[t].y, f00[t].y);
+      const float bx = fmaf(wx[t], f11[t].x - f10[t].x, f10[t].x);
+      const float by = fmaf(wx[t], f11[t].y - f10[t].y, f10[t].y);
+      F = make_float2(fmaf(wy[t], bx - tx, tx), fmaf(wy[t], by - ty, ty));
     }
-    E = fmaf(px.wl[t], l2, E);
+    const float dx = F.x - (xs[t] - xp);
+    const float dy = F.y - (ys[t] - yp);
+    const float r2 = fmaf(dx, dx, dy * dy);
+    const float l = vd_l2_flow(P, r2, fmaf(F.x, F.x, F.y * F.y));
+    E = fmaf(px.wl[t], ob[t] && fr[t] ? l : (ob[t] ? (VD_L_BEHIND / VD_LN2) : 0.0f), E);
   }
   return E;
 }

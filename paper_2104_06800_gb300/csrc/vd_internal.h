@@ -160,6 +160,7 @@ cudaError_t launch_pose_frame(vd_ctx* c, uint32_t itcode, int t);
 cudaError_t launch_pose_score_only(vd_ctx* c);
 // function attributes set once per device before any launch or capture
 cudaError_t vd_pose_prepare(void);
+cudaError_t vd_depth_prepare(void);
 cudaError_t launch_initial_rho(vd_ctx* c);
 cudaError_t launch_eight_point(vd_ctx* c);
 cudaError_t launch_fill(float* p, float v, size_t n, cudaStream_t s);
