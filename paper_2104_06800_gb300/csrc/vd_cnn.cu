@@ -20,8 +20,8 @@
 // tensor-memory accumulators of N columns and commits them to an mbarrier;
 // each warp reads its 32 accumulator lanes with tcgen05.ld.  The backward
 // data gradient is the same GEMM on dL/dz with the weights flipped by 180
-// degrees and transposed; the weight gradient is a float32 reduction over
-// pixels on the CUDA cores, in a fixed order.
+// degrees and transposed; the weight gradient is a GEMM over the pixels of
+// both images (k_wgrad_tc).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -60,29 +60,27 @@ __device__ __forceinline__ uint64_t vd_umma_desc(uint32_t saddr, uint32_t lbo, u
   return d;
 }
 
-// Shared-memory matrix descriptor of a K-major operand in a swizzled layout
-// (rows of `row_bytes` = 32 or 64 bytes, 16-byte chunks permuted by the
-// smem address bits above the row: the layout the tensor copy writes with
-// the same swizzle): SBO = 8 rows, LBO unused (one K step fits a row),
-// swizzle mode 6 (32 B) or 4 (64 B) in bits 61-63; the base-offset field
-// (bits 49-51) carries the start's phase in the pattern when VD_SW_PHASE.
-#ifndef VD_SW_PHASE
-#define VD_SW_PHASE 0
-#endif
-__device__ __forceinline__ uint64_t vd_umma_desc_sw(uint32_t saddr, uint32_t row_bytes) {
+// Shared-memory matrix descriptor of an operand in a swizzled layout (rows of
+// `row_bytes` = 32 or 64 bytes, 16-byte chunks permuted by the smem address
+// bits above the row: the layout the tensor copy writes with the same
+// swizzle): swizzle mode 6 (32 B) or 4 (64 B) in bits 61-63, base offset 0.
+// K-major (a row = one M or N index, K along it): SBO = 8 rows, LBO unused
+// (one K step fits a row).  MN-major (a row = one K index, M or N along it):
+// SBO = 8 rows, LBO = distance of the next row_bytes / 2 M or N indices.
+__device__ __forceinline__ uint64_t vd_umma_desc_sw(uint32_t saddr, uint32_t row_bytes,
+                                                    uint32_t lbo = 16) {
   uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;                                   // LBO (unused)
+  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
   d |= (uint64_t)(((8u * row_bytes) >> 4) & 0x3FFFu) << 32;  // SBO
   d |= (uint64_t)1 << 46;
-  if (VD_SW_PHASE) d |= (uint64_t)((saddr >> 7) & 7u) << 49;
   d |= (uint64_t)(row_bytes == 64 ? 4u : 6u) << 61;
   return d;
 }
 
 // Instruction descriptor of kind::f16: f32 accumulator, bf16 A and B, both
-// K-major, N >> 3 and M >> 4.
-__host__ __device__ constexpr uint32_t vd_idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
+// K-major or (mn) both MN-major (bits 15 and 16), N >> 3 and M >> 4.
+__host__ __device__ constexpr uint32_t vd_idesc_bf16(int M, int N, bool mn = false) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? 3u << 15 : 0u) | ((uint32_t)(N >> 3) << 17) |
          ((uint32_t)(M >> 4) << 24);
 }
 
@@ -157,9 +155,6 @@ __device__ __forceinline__ void vd_bulk_load(uint32_t dst, const void* src, uint
       : "memory");
 }
 
-// Tiled TMA load of one box of a rank-4 tensor map at (c0, c1, c2, c3); c0
-// (the innermost coordinate) must be a multiple of 16 bytes' worth of
-// elements.
 // Tiled TMA load of one box of a rank-3 tensor map at (c0, c1, c2); c0 (the
 // innermost coordinate) must be a multiple of 16 bytes' worth of elements.
 __device__ __forceinline__ void vd_tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0,
@@ -168,16 +163,6 @@ __device__ __forceinline__ void vd_tma_load_3d(uint32_t dst, const CUtensorMap* 
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
       "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(vd_smem_u32(m))
-      : "memory");
-}
-
-__device__ __forceinline__ void vd_tma_load_4d(uint32_t dst, const CUtensorMap* map, int c0,
-                                               int c1, int c2, int c3, uint64_t* m) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3),
-      "r"(vd_smem_u32(m))
       : "memory");
 }
 
@@ -221,6 +206,47 @@ __device__ __forceinline__ void vd_tmem_ld16(uint32_t taddr, float* v) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// 3 C consecutive f32 columns (C = 8 or 16) of this warp's 32 accumulator
+// lanes, the three loads in flight together.
+template <int C>
+__device__ __forceinline__ void vd_tmem_ld3(uint32_t taddr, float* v) {
+  static_assert(C == 8 || C == 16, "columns per load");
+  uint32_t r[3 * C];
+  if constexpr (C == 16) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%48];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%49];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47}, [%50];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+          "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
+          "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]),
+          "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
+          "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]),
+          "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]),
+          "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47])
+        : "r"(taddr), "r"(taddr + 16), "r"(taddr + 32)
+        : "memory");
+  } else {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%24];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%25];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%26];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+          "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
+          "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]),
+          "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23])
+        : "r"(taddr), "r"(taddr + 8), "r"(taddr + 16)
+        : "memory");
+  }
+#pragma unroll
+  for (int i = 0; i < 3 * C; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // ---------------------------------------------------------------------------
@@ -381,7 +407,6 @@ k_conv_tc(const __grid_constant__ CUtensorMap xmap, int Wimg, int Himg, int tile
         // operand at byte offset o has the descriptor + o / 16 (the start
         // field is the shared address / 16, 14 bits, and every address of
         // the CTA's shared memory fits it without a carry)
-        static_assert(VD_SW_PHASE == 0, "offset descriptors need a fixed base-offset field");
         const uint64_t dA0 = vd_umma_desc_sw(a0, S::PIX), dB0 = vd_umma_desc(sB, 128, K * 16);
 #pragma unroll 1
         for (int r = 0; r < R; ++r) {
@@ -610,106 +635,259 @@ __global__ void k_cnn_sum(const double* __restrict__ partial, int n, const int* 
 }
 
 // ---------------------------------------------------------------------------
-// Weight gradient on the CUDA cores: dW[co][tap * CIN + ci] =
+// Weight gradient on the tensor cores: dW[co][tap * CIN + ci] =
 // sum_p dz[p][co] X[p + offset(tap)][ci], db[co] = sum_p dz[p][co].  dz: bf16
 // [HW][COUT]; X: bf16 [HW][CIN].
-// The image is cut into tiles of WG_ROWS rows x WG_COLS pixels; block b
-// takes tiles b, b + gridDim.x, ... in order.  A block stages a tile's
-// input halo and dz in shared memory; thread (co8, ci) holds dW for 8
-// output channels x 9 taps of input channel ci in registers and walks the
-// tile's pixels row by row, sliding its 3 x 3 window of X along the row (3
-// new values, one 16-byte dz load and 72 FMAs per pixel).  The block's sums
-// go to partial[b][co][k] (and partial_b[b][co]); k_cnn_wgrad_reduce adds
-// the blocks in index order, so the result does not depend on scheduling.
+// A GEMM whose K is the pixels of a row and whose operands are both
+// MN-major: in shared memory, as the tensor copy writes them, a pixel is one
+// swizzle row of 32 or 64 bytes and its channels lie along M (dz) or N (X).
+// One MMA takes 16 pixels x .. x + 15 of one row y of X:
+//   N = 3 CIN: the three taps kx are X shifted by one pixel each, the next
+//     CIN columns one pixel (one row) further: LBO = one pixel;
+//   M = 128: rows y - 1, y, y + 1, .. of dz, COUT values each, the next one
+//     row of the dz tile further: LBO = one dz tile row.  dz row y - 1 + j is
+//     tap ky = 2 - j; the rows past j = 2 are never read back.
+// So all nine taps of 16 pixels are one MMA that reads 7 KB (COUT = CIN = 32)
+// of shared memory, against 9 x 5 KB of a tap at a time.
+// A tile is WG_ROWS rows of X by 128 pixels of dz (X with one pixel more on
+// each side, dz with one row more above and below, zeros outside the image).
+// Persistent, warp-specialised like k_conv_tc: warp 0 loads tiles into a ring
+// of WG_STAGES, one thread of warp 1 issues a tile's MMAs in chains of
+// WG_CHAIN into a ring of WG_ACC tensor-memory accumulators, warps 4 to 11
+// (two per lane quarter, half of the columns each) add the tile's dz into db
+// from shared memory and every finished chain into registers, and write the
+// block's sums to partial[b][co][k] and partial_b[b][co]; k_cnn_wgrad_reduce
+// adds the blocks in index order.  The tiles of a block are fixed, so the
+// result does not depend on scheduling.
+// WG_CHAIN: the tensor core truncates its running float32 sum, so a chain's
+// error grows with its length; the registers round to nearest.  Relative
+// error against float64 of a 640 x 480 layer with random data / with data of
+// one sign: chains of a whole tile (32 MMAs) 3.1e-7 / 3.6e-7, of 8 1.4e-7 /
+// 5.4e-8, of 4 1.4e-7 / 5.2e-8, of 2 1.7e-7 / 5.3e-8; the CUDA-core
+// reduction this replaced (a float32 chain per thread) 1.9e-7 / 6.6e-8.  On
+// 166 x 72 pixels 8 is above it (1.11e-7 against 1.03e-7) and 4 is not
+// (9.98e-8), so 4.
+// Bound: the issue of the chains and their waits, about 18 us of the 24 (the
+// operand reads of a 640 x 480 layer take 3.5 us, its 39 MB from HBM 5.8).
+// With the sum over the blocks 33 us per layer of 32 x 32 channels, 166
+// before (142 and 21; 8 output channels x 9 taps per thread).
 // ---------------------------------------------------------------------------
-#ifndef WG_BLOCKS
-#define WG_BLOCKS 608
-#endif
 #define WG_ROWS 4
-#define WG_COLS 64
+#define WG_STAGES 2
+#ifndef WG_CHAIN
+#define WG_CHAIN 4
+#endif
+#define WG_ACC 4
+#define WG_THREADS 384
+#define WG_MAX_BLOCKS 256          // capacity of the partial sums
 
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(COUT / 8 * CIN)
-k_cnn_wgrad(const __nv_bfloat16* __restrict__ X, const __nv_bfloat16* __restrict__ dz, int Wimg,
-            int Himg, float* __restrict__ partial, float* __restrict__ partial_b) {
-  constexpr int K = 9 * CIN, NT = COUT / 8 * CIN;
-  constexpr int HR = WG_ROWS + 2, HC = WG_COLS + 2;
-  __shared__ __align__(16) __nv_bfloat16 sX[HR * HC * CIN];
-  __shared__ __align__(16) __nv_bfloat16 sD[WG_ROWS * WG_COLS * COUT];
-  const int tid = threadIdx.x, ci = tid % CIN, co8 = tid / CIN;
-  const int tiles_x = (Wimg + WG_COLS - 1) / WG_COLS;
-  const int n_tiles = tiles_x * ((Himg + WG_ROWS - 1) / WG_ROWS);
-  float acc[8][9];
-#pragma unroll
-  for (int c = 0; c < 8; ++c)
-#pragma unroll
-    for (int t = 0; t < 9; ++t) acc[c][t] = 0.0f;
-  float accb = 0.0f;
-  for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const int y0 = tile / tiles_x * WG_ROWS, x0 = tile % tiles_x * WG_COLS;
-    __syncthreads();   // the previous tile's values are no longer read
-    for (int i = tid; i < HR * HC * (CIN / 8); i += NT) {   // pixels fastest: coalesced
-      const int g = i / (HR * HC), px = i - g * (HR * HC);
-      const int yy = y0 - 1 + px / HC, xx = x0 - 1 + px % HC;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (yy >= 0 && yy < Himg && xx >= 0 && xx < Wimg)
-        v = *reinterpret_cast<const uint4*>(X + ((size_t)yy * Wimg + xx) * CIN + 8 * g);
-      *reinterpret_cast<uint4*>(sX + (size_t)px * CIN + 8 * g) = v;
+struct VdWgradShape {
+  static constexpr uint32_t PX = (uint32_t)CIN * 2, PD = (uint32_t)COUT * 2;   // bytes of a pixel
+  static constexpr uint32_t X_BOX = (uint32_t)WG_ROWS * CNN_HALO_X * PX;
+  static constexpr uint32_t D_ROW = (uint32_t)CNN_TILE * PD;
+  static constexpr uint32_t D_BOX = (uint32_t)(WG_ROWS + 2) * D_ROW;
+  // M = 128 reaches 128 / COUT rows down from the last row of X
+  static constexpr uint32_t D_ALL = (uint32_t)(WG_ROWS - 1 + 128 / COUT) * D_ROW;
+  static constexpr uint32_t D_OFF = vd_round1024(X_BOX);
+  static constexpr uint32_t STAGE = vd_round1024(D_OFF + D_ALL);
+  static constexpr uint32_t SMEM = WG_STAGES * STAGE + 1024;
+  static constexpr int N = 3 * CIN;
+};
+
+// Rows and 16-pixel steps of a tile inside the image (the others are zeros).
+__device__ __forceinline__ int wg_rows(int tile, int tiles_x, int Himg) {
+  return min(WG_ROWS, Himg - tile / tiles_x * WG_ROWS);
+}
+__device__ __forceinline__ int wg_steps(int tile, int tiles_x, int Wimg) {
+  return min(CNN_TILE / 16, (Wimg - tile % tiles_x * CNN_TILE + 15) / 16);
+}
+
+template <int CIN, int COUT>
+__global__ void __launch_bounds__(WG_THREADS, 1)
+k_wgrad_tc(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap dmap,
+           int Wimg, int Himg, int tiles_x, int n_tiles, float* __restrict__ partial,
+           float* __restrict__ partial_b, int* __restrict__ err) {
+  using S = VdWgradShape<CIN, COUT>;
+  constexpr int N = S::N, K = 9 * CIN, NS = WG_STAGES, CH = COUT / 8;
+  static_assert(S::SMEM <= 232448 && S::D_ALL >= S::D_BOX, "tile");
+  extern __shared__ uint8_t smem[];
+  __shared__ uint64_t full[NS], empty[NS], accfull[WG_ACC], accempty[WG_ACC], fin;
+  __shared__ uint32_t tmem_base;
+  __shared__ int s_abort;
+  __shared__ float s_b[256][9];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  volatile int* abort = &s_abort;
+  if (warp == 2) vd_tmem_alloc(&tmem_base, 512);
+  if (tid == 32) {
+    for (int s = 0; s < NS; ++s) {
+      vd_mbar_init(&full[s], 1);
+      vd_mbar_init(&empty[s], 1 + 8);      // the MMAs' commit and the eight db warps
     }
-    for (int i = tid; i < WG_ROWS * WG_COLS * (COUT / 8); i += NT) {
-      const int g = i / (WG_ROWS * WG_COLS), px = i - g * (WG_ROWS * WG_COLS);
-      const int yy = y0 + px / WG_COLS, xx = x0 + px % WG_COLS;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (yy < Himg && xx < Wimg)
-        v = *reinterpret_cast<const uint4*>(dz + ((size_t)yy * Wimg + xx) * COUT + 8 * g);
-      *reinterpret_cast<uint4*>(sD + (size_t)px * COUT + 8 * g) = v;
+    for (int a = 0; a < WG_ACC; ++a) {
+      vd_mbar_init(&accfull[a], 1);
+      vd_mbar_init(&accempty[a], 8);
     }
-    __syncthreads();
-#pragma unroll 1
-    for (int r = 0; r < WG_ROWS; ++r) {
-      float w[3][3];   // X at rows r .. r + 2, columns x .. x + 2 of the halo
-#pragma unroll
-      for (int dy = 0; dy < 3; ++dy) {
-        w[dy][0] = __bfloat162float(sX[((r + dy) * HC + 0) * CIN + ci]);
-        w[dy][1] = __bfloat162float(sX[((r + dy) * HC + 1) * CIN + ci]);
+    vd_mbar_init(&fin, 1);
+    s_abort = 0;
+  }
+  vd_tc_fence_before();
+  __syncthreads();
+  vd_tc_fence_after();
+  const uint32_t dt = tmem_base;
+  const uint32_t s0 = (vd_smem_u32(smem) + 1023u) & ~1023u;
+  const int my_tiles = blockIdx.x < n_tiles ? (n_tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  if (warp == 0) {
+    if (lane == 0) {   // producer
+      int issued = 0;
+      for (int i = 0; i < my_tiles && !*abort; ++i) {
+        const int s = i % NS;
+        if (i >= NS && !vd_mbar_wait_or_abort(&empty[s], ((i / NS) - 1) & 1, abort)) {
+          atomicExch(err, 1);
+          *abort = 1;
+          break;
+        }
+        const int tile = blockIdx.x + i * gridDim.x;
+        const int x0 = (tile % tiles_x) * CNN_TILE, y0 = (tile / tiles_x) * WG_ROWS;
+        vd_mbar_expect_tx(&full[s], S::X_BOX + S::D_BOX);
+        vd_tma_load_3d(s0 + s * S::STAGE, &xmap, 0, x0 - 1, y0, &full[s]);
+        vd_tma_load_3d(s0 + s * S::STAGE + S::D_OFF, &dmap, 0, x0, y0 - 1, &full[s]);
+        issued = i + 1;
       }
-#pragma unroll 2
-      for (int x = 0; x < WG_COLS; ++x) {
+      // the loads in flight land before the CTA ends
+      for (int i = issued > NS ? issued - NS : 0; i < issued; ++i)
+        vd_mbar_wait_bounded(&full[i % NS], (i / NS) & 1);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {   // MMA issuer
+      bool any = false;
+      constexpr uint32_t idesc = vd_idesc_bf16(128, N, true);
+      int q = 0;                         // chains so far
+      for (int i = 0; i < my_tiles && !*abort; ++i) {
+        const int s = i % NS;
+        bool ok = vd_mbar_wait_or_abort(&full[s], (i / NS) & 1, abort);
+        vd_tc_fence_after();
+        const int tile = blockIdx.x + i * gridDim.x;
+        const int nk = wg_steps(tile, tiles_x, Wimg), n = nk * wg_rows(tile, tiles_x, Himg);
+        const uint32_t sx = s0 + s * S::STAGE;
+        // descriptors of the row and of the 16-pixel step (start field: address / 16)
+        uint64_t dAr = vd_umma_desc_sw(sx + S::D_OFF, S::PD, S::D_ROW), dAk = dAr;
+        uint64_t dBr = vd_umma_desc_sw(sx, S::PX, S::PX), dBk = dBr;
+        int k = 0;
+        for (int c0 = 0; ok && c0 < n; c0 += WG_CHAIN, ++q) {
+          const int a = q % WG_ACC;
+          if (q >= WG_ACC) {
+            ok = vd_mbar_wait_or_abort(&accempty[a], ((q / WG_ACC) - 1) & 1, abort);
+            if (!ok) break;
+            vd_tc_fence_after();
+          }
 #pragma unroll
-        for (int dy = 0; dy < 3; ++dy)
-          w[dy][2] = __bfloat162float(sX[((r + dy) * HC + x + 2) * CIN + ci]);
-        const __nv_bfloat16* d = sD + (size_t)(r * WG_COLS + x) * COUT + co8 * 8;
-        const uint4 dv = *reinterpret_cast<const uint4*>(d);
-        const __nv_bfloat162* d2 = reinterpret_cast<const __nv_bfloat162*>(&dv);
-        float dzv[8];
+          for (int c = 0; c < WG_CHAIN; ++c) {
+            if (c0 + c >= n) break;
+            vd_umma_bf16(dt + a * 128, dAk, dBk, idesc, c ? 1u : 0u);
+            dAk += (16 * S::PD) >> 4;    // the next 16 pixels, or the next row
+            dBk += (16 * S::PX) >> 4;
+            if (++k == nk) {
+              k = 0;
+              dAr += S::D_ROW >> 4;
+              dBr += (CNN_HALO_X * S::PX) >> 4;
+              dAk = dAr;
+              dBk = dBr;
+            }
+          }
+          vd_umma_commit(&accfull[a]);
+          any = true;
+        }
+        if (!ok) {
+          atomicExch(err, 1);
+          *abort = 1;
+          break;
+        }
+        vd_umma_commit(&empty[s]);
+      }
+      if (any) {   // every MMA issued has finished before the memory is freed
+        vd_umma_commit(&fin);
+        vd_mbar_wait_bounded(&fin, 0);
+      }
+    }
+  } else if (warp >= 4) {
+    const int quarter = warp & 3, part = (warp - 4) >> 2, et = tid - 128;
+    // accumulator lane m = 32 quarter + lane holds dz row slot m / COUT
+    const int m = 32 * quarter + lane, slot = m / COUT, co = m % COUT;
+    const bool used = 32 * quarter < 3 * COUT;   // warp-uniform
+    const uint32_t tl = dt + ((uint32_t)(quarter * 32) << 16) + part * (N / 2);
+    float acc[N / 2];
+#pragma unroll
+    for (int c = 0; c < N / 2; ++c) acc[c] = 0.0f;
+    // db: thread et sums channels 8 ch .. 8 ch + 7 of pixels px0, px0 + 256 / CH, ..
+    const int ch = et % CH, px0 = et / CH;
+    float b[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) b[c] = 0.0f;
+    int q = 0, ok = 1;
+    for (int i = 0; i < my_tiles && ok; ++i) {
+      const int s = i % NS;
+      if (lane == 0) ok = vd_mbar_wait_or_abort(&full[s], (i / NS) & 1, abort) ? 1 : 0;
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      if (!ok) break;
+      // every lane acquires the phase itself before it reads the tile
+      vd_mbar_try_wait(&full[s], (i / NS) & 1);
+      const uint8_t* d = smem + (s0 - vd_smem_u32(smem)) + s * S::STAGE + S::D_OFF + S::D_ROW;
+#pragma unroll 4
+      for (int p = px0; p < WG_ROWS * CNN_TILE; p += 256 / CH) {   // rows y0 .. y0 + WG_ROWS - 1
+        const int sw = COUT == 32 ? (p >> 1) & 3 : (p >> 2) & 1;
+        const uint4 v = *reinterpret_cast<const uint4*>(d + (size_t)p * S::PD + 16 * (ch ^ sw));
+        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          const float2 f = __bfloat1622float2(d2[c]);
-          dzv[2 * c] = f.x;
-          dzv[2 * c + 1] = f.y;
-        }
-        accb += __bfloat162float(d[ci & 7]);
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-#pragma unroll
-          for (int dy = 0; dy < 3; ++dy)
-#pragma unroll
-            for (int dx = 0; dx < 3; ++dx)
-              acc[c][dy * 3 + dx] = fmaf(dzv[c], w[dy][dx], acc[c][dy * 3 + dx]);
-#pragma unroll
-        for (int dy = 0; dy < 3; ++dy) {
-          w[dy][0] = w[dy][1];
-          w[dy][1] = w[dy][2];
+          const float2 f = __bfloat1622float2(h[c]);
+          b[2 * c] += f.x;
+          b[2 * c + 1] += f.y;
         }
       }
+      __syncwarp();
+      if (lane == 0) vd_mbar_arrive(&empty[s]);
+      const int tile = blockIdx.x + i * gridDim.x;
+      const int n = wg_steps(tile, tiles_x, Wimg) * wg_rows(tile, tiles_x, Himg);
+      for (int c0 = 0; c0 < n; c0 += WG_CHAIN, ++q) {
+        const int a = q % WG_ACC;
+        if (lane == 0) ok = vd_mbar_wait_or_abort(&accfull[a], (q / WG_ACC) & 1, abort) ? 1 : 0;
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok) break;
+        vd_tc_fence_after();
+        if (used) {
+          float v[N / 2];
+          vd_tmem_ld3<N / 6>(tl + a * 128, v);
+#pragma unroll
+          for (int c = 0; c < N / 2; ++c) acc[c] += v[c];
+        }
+        vd_tc_fence_before();
+        __syncwarp();
+        if (lane == 0) vd_mbar_arrive(&accempty[a]);
+      }
     }
+    if (!ok && lane == 0) {
+      atomicExch(err, 1);
+      *abort = 1;
+    }
+    if (slot < 3) {   // column kx CIN + ci is tap (2 - slot, kx)
+      float* out = partial + ((size_t)blockIdx.x * COUT + co) * K + (2 - slot) * 3 * CIN +
+                   part * (N / 2);
+#pragma unroll
+      for (int c = 0; c < N / 2; c += 4)
+        *reinterpret_cast<float4*>(out + c) = make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) s_b[et][c] = b[c];
   }
-  float* out = partial + (size_t)blockIdx.x * COUT * K;
-#pragma unroll
-  for (int c = 0; c < 8; ++c)
-#pragma unroll
-    for (int t = 0; t < 9; ++t) out[(size_t)(co8 * 8 + c) * K + t * CIN + ci] = acc[c][t];
-  if (ci < 8) partial_b[blockIdx.x * COUT + co8 * 8 + ci] = accb;
+  vd_tc_fence_before();
+  __syncthreads();
+  if (warp == 2) vd_tmem_dealloc(dt, 512);
+  if (tid < COUT) {   // channel tid: the threads of its chunk in order
+    float t = 0.0f;
+    for (int k = tid / 8; k < 256; k += CH) t += s_b[k][tid % 8];
+    partial_b[blockIdx.x * COUT + tid] = t;
+  }
 }
 
 // Sum of the blocks' partials.  The partials hold `stride` values per block
@@ -858,22 +1036,23 @@ static PFN_cuTensorMapEncodeTiled_v12000 vd_encode_tiled() {
   return fn;
 }
 
-// Tensor map of a bf16 image with cin = 16 or 32 channels per pixel
-// ([H][W][cin]): dims {cin, W, H}, box {cin, 130, rows + 2}, zero fill
-// outside the image, 32- or 64-byte swizzle (one pixel is one swizzle row,
-// the layout vd_umma_desc_sw reads).
-static cudaError_t vd_halo_map(CUtensorMap* m, const void* X, int cin, int W, int H, int rows) {
+// Tensor map of a bf16 image with ch = 16 or 32 channels per pixel
+// ([H][W][ch]): dims {ch, W, H}, box {ch, bx, by}, zero fill outside the
+// image, 32- or 64-byte swizzle (one pixel is one swizzle row, the layout
+// vd_umma_desc_sw reads).
+static cudaError_t vd_image_map(CUtensorMap* m, const void* X, int ch, int W, int H, int bx,
+                                int by) {
   const PFN_cuTensorMapEncodeTiled_v12000 enc = vd_encode_tiled();
   if (!enc) return cudaErrorNotSupported;
-  if ((reinterpret_cast<uintptr_t>(X) & 15u) || (cin != 16 && cin != 32))
+  if ((reinterpret_cast<uintptr_t>(X) & 15u) || (ch != 16 && ch != 32))
     return cudaErrorInvalidValue;
-  const cuuint64_t dims[3] = {(cuuint64_t)cin, (cuuint64_t)W, (cuuint64_t)H};
-  const cuuint64_t strides[2] = {(cuuint64_t)cin * 2, (cuuint64_t)W * cin * 2};
-  const cuuint32_t box[3] = {(cuuint32_t)cin, CNN_HALO_X, (cuuint32_t)rows + 2};
+  const cuuint64_t dims[3] = {(cuuint64_t)ch, (cuuint64_t)W, (cuuint64_t)H};
+  const cuuint64_t strides[2] = {(cuuint64_t)ch * 2, (cuuint64_t)W * ch * 2};
+  const cuuint32_t box[3] = {(cuuint32_t)ch, (cuuint32_t)bx, (cuuint32_t)by};
   const cuuint32_t es[3] = {1, 1, 1};
   const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(X), dims,
                          strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                         cin == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+                         ch == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
@@ -900,7 +1079,7 @@ static cudaError_t launch_conv(const __nv_bfloat16* X, int W, int H, const __nv_
     slots = sms * per_sm;
   }
   CUtensorMap map;
-  cudaError_t e = vd_halo_map(&map, X, K / 9, W, H, R);
+  cudaError_t e = vd_image_map(&map, X, K / 9, W, H, CNN_HALO_X, R + 2);
   if (e != cudaSuccess) return e;
   if (reinterpret_cast<uintptr_t>(Wt) & 15u) return cudaErrorInvalidValue;
   const int tiles_x = (W + CNN_TILE - 1) / CNN_TILE;
@@ -951,14 +1130,30 @@ static cudaError_t cnn_forward(vd_cnn* n, const float* flow, int W, int H, cudaS
 template <int CIN, int COUT>
 static cudaError_t launch_wgrad(vd_cnn* n, int l, const __nv_bfloat16* dz, int W, int H,
                                 cudaStream_t s) {
-  k_cnn_wgrad<CIN, COUT><<<WG_BLOCKS, COUT / 8 * CIN, 0, s>>>(n->act[l], dz, W, H,
-                                                                   n->wg_partial,
-                                                                   n->wg_partial_b);
-  cudaError_t e = cudaGetLastError();
+  using S = VdWgradShape<CIN, COUT>;
+  auto kern = k_wgrad_tc<CIN, COUT>;
+  static int slots = 0;   // persistent grid: one CTA per SM (set up once)
+  if (!slots) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+    if (e != cudaSuccess) return e;
+    slots = min(sms, WG_MAX_BLOCKS);
+  }
+  CUtensorMap xmap, dmap;
+  cudaError_t e = vd_image_map(&xmap, n->act[l], CIN, W, H, CNN_HALO_X, WG_ROWS);
+  if (e == cudaSuccess) e = vd_image_map(&dmap, dz, COUT, W, H, CNN_TILE, WG_ROWS + 2);
   if (e != cudaSuccess) return e;
+  const int tiles_x = (W + CNN_TILE - 1) / CNN_TILE;
+  const int n_tiles = tiles_x * ((H + WG_ROWS - 1) / WG_ROWS), nblk = min(n_tiles, slots);
+  kern<<<nblk, WG_THREADS, S::SMEM, s>>>(xmap, dmap, W, H, tiles_x, n_tiles, n->wg_partial,
+                                         n->wg_partial_b, n->err);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int stride = COUT * 9 * CIN, nout = n->cout[l] * 9 * CIN;
   k_cnn_wgrad_reduce<<<(nout + 31) / 32, 256, 0, s>>>(
-      n->wg_partial, n->wg_partial_b, WG_BLOCKS, stride, nout, COUT, n->cout[l],
+      n->wg_partial, n->wg_partial_b, nblk, stride, nout, COUT, n->cout[l],
       n->grad + n->woff[l], n->grad + n->boff[l]);
   return cudaGetLastError();
 }
@@ -1088,8 +1283,8 @@ extern "C" vd_status vd_cnn_create(int n_flows, unsigned long long seed, vd_cnn*
       e = cudaMalloc(&n->wd[l], sizeof(__nv_bfloat16) * n->cin[l] * 9 * npad);
   }
   if (e == cudaSuccess)
-    e = cudaMalloc(&n->wg_partial, sizeof(float) * WG_BLOCKS * CNN_WIDTH * 9 * CNN_WIDTH);
-  if (e == cudaSuccess) e = cudaMalloc(&n->wg_partial_b, sizeof(float) * WG_BLOCKS * CNN_WIDTH);
+    e = cudaMalloc(&n->wg_partial, sizeof(float) * WG_MAX_BLOCKS * CNN_WIDTH * 9 * CNN_WIDTH);
+  if (e == cudaSuccess) e = cudaMalloc(&n->wg_partial_b, sizeof(float) * WG_MAX_BLOCKS * CNN_WIDTH);
   if (e == cudaSuccess) e = cudaMalloc(&n->loss, sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&n->nmask, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&n->err, sizeof(int));
