@@ -4,12 +4,13 @@
 // confidence weights, solved by Levenberg-Marquardt; covariance (J^T J)^-1.
 //
 // The device evaluates, at a given (T, s), the energy and the normal
-// equations of every associated pixel of keyframe 2: k_ka_normals computes
-// depth map 1's normals once, k_ka_accum sums E, H (upper triangle of 7 x 7)
-// and g per block over a fixed pixel range (float64 per pixel, warp
-// butterflies and a fixed warp order within the block), k_ka_sum adds the
+// equations of every associated pixel of keyframe 2: k_ka_rays and
+// k_ka_normals prepare the rays and depth map 1's normals once, k_ka_accum
+// sums E, H (upper triangle of 7 x 7) and g per block over a fixed pixel
+// range (float64 per pixel, a fixed order within the block), k_ka_sum adds the
 // blocks in index order.  The host runs the Levenberg-Marquardt schedule on
-// the 37 sums of each evaluation.
+// the sums of each evaluation.
+#include <algorithm>
 #include <cmath>
 #include <utility>
 
@@ -17,9 +18,9 @@
 #include "vd_geom64.cuh"
 
 #define KA_BLOCK 256
-#define KA_NS 37          // E, H (28), g (7), n
-#define KA_KINK 0.2       // no normal where a second difference exceeds this of the span
-#define KA_GATE 0.2       // a pair counts when the depths agree within this fraction
+#define KA_NS 37             // E, H (28), g (7), n
+#define KA_KINK 0.2          // no normal where a second difference exceeds this of the span
+#define KA_GATE 0.2          // a pair counts when the depths agree within this fraction
 #define KA_LAMBDA0 1e-3
 #define KA_STEP_TOL 1e-10
 
@@ -28,11 +29,43 @@ struct KaCam {
   int W, H;
 };
 
+struct KaPose {
+  double T[12];
+};
+
 struct __align__(16) KaNormal {   // unit normal and a validity flag w
   double x, y, z, w;
 };
 
 __device__ __forceinline__ bool ka_valid(float t) { return isfinite(t) && t > 0.0f; }
+
+// The reciprocal of a normal x > 0 to about one unit in the last place: the
+// hardware's float64 seed (some 20 bits) and two Newton steps, each squaring
+// the relative error.
+__device__ __forceinline__ double ka_rcp(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+
+// a / b from r = ka_rcp(b), correctly rounded: the quotient a r corrected by
+// its exact remainder (P. Markstein, IBM J. Res. Dev. 34(1), 1990).  What is
+// rounded last lies within 2^-51 units in the last place of a / b, so that
+// the result is that of the division unless a / b is that close to a
+// midpoint.  Divisions by one value share its reciprocal: three operations
+// each instead of a division sequence.
+__device__ __forceinline__ double ka_div(double a, double b, double r) {
+  const double q = a * r;
+  return fma(fma(-b, q, a), r, q);
+}
+
+// The rays' components of every column and row.
+__global__ void k_ka_rays(KaCam c, double* __restrict__ rx, double* __restrict__ ry) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < c.W) rx[i] = ((double)i - c.cx) / c.fx;
+  if (i < c.H) ry[i] = ((double)i - c.cy) / c.fy;
+}
 
 __device__ __forceinline__ void ka_point(const KaCam& c, const float* th, int u, int v,
                                          double* P) {
@@ -89,86 +122,139 @@ k_ka_normals(const float* __restrict__ theta1, KaCam c, KaNormal* __restrict__ n
   n1[j] = out;
 }
 
-// Block b sums pixels [b per, (b+1) per) of keyframe 2 into partial[b][37]:
-// E, H_ik (i <= k, row by row), g_i, n.  Ts: T (12) at the evaluation.
+// One evaluation at (T, s).  Block b sums the pixels [b per, (b + 1) per) of
+// keyframe 2 into partial[b][37]: E, H_ik (i <= k, row by row), g_i, n; with
+// FULL false only E and n (the same E).  Bound: the float64 pipe, two
+// operations per SM and clock: some 190 a pixel (90 with FULL false) are 135
+// us of a 1216 x 368 pair, and 163 (80) are measured.  With a division
+// sequence per division and a butterfly per sum (330 operations a pixel and
+// 185 additions a thread) it took 274.
+template <bool FULL>
 __global__ void __launch_bounds__(KA_BLOCK)
 k_ka_accum(const float* __restrict__ theta1, const KaNormal* __restrict__ n1,
            const float* __restrict__ theta2, const float* __restrict__ conf2, KaCam c,
-           const double* __restrict__ Ts, double s, double cc, double* __restrict__ partial) {
-  __shared__ double sT[12];
-  __shared__ double sW[KA_BLOCK / 32][KA_NS];
-  if (threadIdx.x < 12) sT[threadIdx.x] = Ts[threadIdx.x];
-  __syncthreads();
+           const double* __restrict__ rx, const double* __restrict__ ry, KaPose Tp, double s,
+           double cc, double* __restrict__ partial) {
+  constexpr int NA = FULL ? 36 : 1;               // float64 sums: E, H, g
+  constexpr int NP = FULL ? 40 : 1;               // padded for the halvings below
+  __shared__ double sW[KA_BLOCK / 32][NP];
+  __shared__ int sN[KA_BLOCK / 32];
   const size_t npix = (size_t)c.W * c.H;
   const size_t per = (npix + gridDim.x - 1) / gridDim.x;
   const size_t beg = min(npix, (size_t)blockIdx.x * per), end = min(npix, beg + per);
-  double acc[KA_NS];
+  // nonnegative doubles order like their bit patterns, and a negative one or
+  // a NaN is above them: one unsigned compare is 0 <= x <= W - 1
+  const unsigned long long xmax = (unsigned long long)__double_as_longlong((double)(c.W - 1));
+  const unsigned long long ymax = (unsigned long long)__double_as_longlong((double)(c.H - 1));
+  const double icc = ka_rcp(cc);
+  const double* sT = Tp.T;
+  double acc[NP];
+  int n = 0;
 #pragma unroll
-  for (int i = 0; i < KA_NS; ++i) acc[i] = 0.0;
+  for (int i = 0; i < NP; ++i) acc[i] = 0.0;
   for (size_t j = beg + threadIdx.x; j < end; j += KA_BLOCK) {
     const float t2 = theta2[j];
     if (!ka_valid(t2)) continue;
     const int v = (int)(j / c.W), u = (int)(j - (size_t)v * c.W);
-    const double X[3] = {(double)t2 * (((double)u - c.cx) / c.fx),
-                         (double)t2 * (((double)v - c.cy) / c.fy), (double)t2};
+    const double X[3] = {(double)t2 * rx[u], (double)t2 * ry[v], (double)t2};
     double P[3];
+#pragma unroll
     for (int i = 0; i < 3; ++i)
       P[i] = X[0] * sT[4 * i] + X[1] * sT[4 * i + 1] + X[2] * sT[4 * i + 2] + sT[4 * i + 3];
     if (!(P[2] > (double)VD_Z_EPS)) continue;
-    const double Z = P[2];
-    const double x = c.fx * P[0] / Z + c.cx, y = c.fy * P[1] / Z + c.cy;
-    if (!(x >= 0.0 && x <= (double)(c.W - 1) && y >= 0.0 && y <= (double)(c.H - 1))) continue;
-    const int lu = (int)floor(x + 0.5), lv = (int)floor(y + 0.5);
+    const double Z = P[2], iZ = ka_rcp(Z);
+    const double x = ka_div(c.fx * P[0], Z, iZ) + c.cx, y = ka_div(c.fy * P[1], Z, iZ) + c.cy;
+    if ((unsigned long long)__double_as_longlong(x) > xmax ||
+        (unsigned long long)__double_as_longlong(y) > ymax)
+      continue;
+    // floor(x + 1/2): adding 2^52 rounded down leaves the integer in the low word
+    const int lu = __double2loint(__dadd_rd(x + 0.5, 4503599627370496.0));
+    const int lv = __double2loint(__dadd_rd(y + 0.5, 4503599627370496.0));
     const size_t l = (size_t)lv * c.W + lu;
-    const KaNormal n = n1[l];
-    const float t1 = theta1[l];
-    if (!(n.w > 0.0) || !ka_valid(t1)) continue;
-    const double D = s * (double)t1;
+    const KaNormal m = n1[l];
+    if (!(m.w > 0.0)) continue;                    // (its depth is then valid)
+    const double D = s * (double)theta1[l];
     if (!(fabs(Z - D) <= KA_GATE * D)) continue;   // occlusion gate
-    const double rl[3] = {((double)lu - c.cx) / c.fx, ((double)lv - c.cy) / c.fy, 1.0};
-    const double A = n.x * rl[0] + n.y * rl[1] + n.z * rl[2];
-    const double B = n.x * P[0] + n.y * P[1] + n.z * P[2];
-    const double r = A / Z - B / (D * Z);
+    const double rl[3] = {rx[lu], ry[lv], 1.0};
+    const double A = m.x * rl[0] + m.y * rl[1] + m.z * rl[2];
+    const double B = m.x * P[0] + m.y * P[1] + m.z * P[2];
+    const double DZ = D * Z, iDZ = ka_rcp(DZ), BDZ = ka_div(B, DZ, iDZ);
+    const double r = ka_div(A, Z, iZ) - BDZ;
     const double C = conf2 ? (double)conf2[j] : 1.0;
-    const double q = r / cc;
-    const double w = C / (1.0 + q * q);
+    const double q = ka_div(r, cc, icc);
     acc[0] += C * (0.5 * cc * cc * log1p(q * q));
-    // J = d r / d(omega, v, log s)
-    double g3[3] = {-n.x / (D * Z), -n.y / (D * Z), -n.z / (D * Z)};
-    g3[2] += (B - A * D) / (D * Z * Z);
-    const double J[7] = {P[1] * g3[2] - P[2] * g3[1], P[2] * g3[0] - P[0] * g3[2],
-                         P[0] * g3[1] - P[1] * g3[0], g3[0], g3[1], g3[2], B / (D * Z)};
-    int q2 = 1;
+    ++n;
+    if constexpr (FULL) {
+      const double q1 = 1.0 + q * q;
+      const double w = ka_div(C, q1, ka_rcp(q1));
+      // J = d r / d(omega, v, log s)
+      double g3[3] = {ka_div(-m.x, DZ, iDZ), ka_div(-m.y, DZ, iDZ), ka_div(-m.z, DZ, iDZ)};
+      const double DZZ = DZ * Z;
+      g3[2] += ka_div(B - A * D, DZZ, ka_rcp(DZZ));
+      const double J[7] = {P[1] * g3[2] - P[2] * g3[1], P[2] * g3[0] - P[0] * g3[2],
+                           P[0] * g3[1] - P[1] * g3[0], g3[0], g3[1], g3[2], BDZ};
+      int q2 = 1;
 #pragma unroll
-    for (int i = 0; i < 7; ++i)
+      for (int i = 0; i < 7; ++i)
 #pragma unroll
-      for (int k = i; k < 7; ++k) acc[q2++] += w * J[i] * J[k];
+        for (int k = i; k < 7; ++k) acc[q2++] += w * J[i] * J[k];
 #pragma unroll
-    for (int i = 0; i < 7; ++i) acc[29 + i] += w * J[i] * r;
-    acc[36] += 1.0;
+      for (int i = 0; i < 7; ++i) acc[29 + i] += w * J[i] * r;
+    }
   }
+  // warp sums, every one the tree of an xor butterfly.  FULL: three halvings
+  // (lane bits 4, 3, 2: the upper lanes keep the upper half of the sums and
+  // receive their partner's copy of it) leave five sums a lane, then two
+  // butterflies: 45 float64 additions a lane, not 185
   const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
+  if constexpr (FULL) {
 #pragma unroll
-  for (int i = 0; i < KA_NS; ++i) {
-    double v = acc[i];
+    for (int h = 20, b = 16; h >= 5; h >>= 1, b >>= 1) {
+      const bool upper = (lane & b) != 0;
+#pragma unroll
+      for (int i = 0; i < h; ++i) {
+        const double send = upper ? acc[i] : acc[i + h];
+        const double keep = upper ? acc[i + h] : acc[i];
+        acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, b);
+      }
+    }
+    // lanes with bits 4, 3, 2 = (a, b, c) hold sums 20 a + 10 b + 5 c + 0..4
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      double v = acc[i];
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      if ((lane & 3) == 0) sW[wq][5 * (lane >> 2) + i] = v;
+    }
+  } else {
+    double v = acc[0];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) sW[wq][i] = v;
+    if (lane == 0) sW[wq][0] = v;
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+  if (lane == 0) sN[wq] = n;
   __syncthreads();
-  if (threadIdx.x < KA_NS) {
+  double* out = partial + (size_t)blockIdx.x * KA_NS;
+  if (threadIdx.x < NA) {
     double v = 0.0;
     for (int k = 0; k < KA_BLOCK / 32; ++k) v += sW[k][threadIdx.x];
-    partial[(size_t)blockIdx.x * KA_NS + threadIdx.x] = v;
+    out[threadIdx.x] = v;
+  } else if (threadIdx.x == KA_NS - 1) {
+    int k = 0;
+    for (int i = 0; i < KA_BLOCK / 32; ++i) k += sN[i];
+    out[KA_NS - 1] = (double)k;
   }
 }
 
-// Block i adds sum i over the partials: thread t takes blocks t, t + 256, ...
-// in order, then a fixed tree over the threads.
+// Block i adds sum i (with `full` 0: E and n, i = 0 and 36) over the
+// partials: thread t takes blocks t, t + 256, ... in order, then a fixed tree
+// over the threads.
 __global__ void __launch_bounds__(KA_BLOCK)
-k_ka_sum(const double* __restrict__ partial, int nblk, double* __restrict__ out) {
+k_ka_sum(const double* __restrict__ partial, int nblk, int full, double* __restrict__ out) {
   __shared__ double sv[KA_BLOCK];
-  const int i = blockIdx.x;
+  const int i = full || blockIdx.x == 0 ? blockIdx.x : KA_NS - 1;
   double v = 0.0;
   for (int b = threadIdx.x; b < nblk; b += KA_BLOCK) v += partial[(size_t)b * KA_NS + i];
   sv[threadIdx.x] = v;
@@ -196,28 +282,34 @@ struct KaRun {
   double cc;
   cudaStream_t st;
   KaNormal* n1;
-  double* partial;
-  double* sums;
-  double* Tdev;
+  double *rx, *ry, *partial, *sums;
   int nblk;
 };
 
-cudaError_t ka_eval(const KaRun& k, const double* T, double s, KaEval* out) {
-  cudaError_t e = cudaMemcpyAsync(k.Tdev, T, sizeof(double) * 12, cudaMemcpyHostToDevice, k.st);
+// E and n at (T, s), and (full) the normal equations.
+cudaError_t ka_eval(const KaRun& k, const double* T, double s, bool full, KaEval* out) {
+  KaPose p;
+  for (int i = 0; i < 12; ++i) p.T[i] = T[i];
+  if (full)
+    k_ka_accum<true><<<k.nblk, KA_BLOCK, 0, k.st>>>(k.th1, k.n1, k.th2, k.conf2, k.cam, k.rx, k.ry,
+                                                    p, s, k.cc, k.partial);
+  else
+    k_ka_accum<false><<<k.nblk, KA_BLOCK, 0, k.st>>>(k.th1, k.n1, k.th2, k.conf2, k.cam, k.rx,
+                                                     k.ry, p, s, k.cc, k.partial);
+  k_ka_sum<<<full ? KA_NS : 2, KA_BLOCK, 0, k.st>>>(k.partial, k.nblk, full, k.sums);
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_ka_accum<<<k.nblk, KA_BLOCK, 0, k.st>>>(k.th1, k.n1, k.th2, k.conf2, k.cam, k.Tdev, s, k.cc,
-                                            k.partial);
-  k_ka_sum<<<KA_NS, KA_BLOCK, 0, k.st>>>(k.partial, k.nblk, k.sums);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   double h[KA_NS];
   e = cudaMemcpyAsync(h, k.sums, sizeof h, cudaMemcpyDeviceToHost, k.st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(k.st);
   if (e != cudaSuccess) return e;
   out->E = h[0];
-  for (int i = 0, q = 1; i < 7; ++i)
-    for (int j = i; j < 7; ++j, ++q) out->H[7 * i + j] = out->H[7 * j + i] = h[q];
-  for (int i = 0; i < 7; ++i) out->g[i] = h[29 + i];
   out->n = (long long)h[36];
+  if (full) {
+    for (int i = 0, q = 1; i < 7; ++i)
+      for (int j = i; j < 7; ++j, ++q) out->H[7 * i + j] = out->H[7 * j + i] = h[q];
+    for (int i = 0; i < 7; ++i) out->g[i] = h[29 + i];
+  }
   return cudaSuccess;
 }
 
@@ -271,18 +363,21 @@ extern "C" vd_status vd_ka_align(const float* depth1, const float* depth2, const
   k.th1 = depth1;
   k.th2 = depth2;
   k.conf2 = conf2;
-  k.cam = KaCam{K[0], K[1], K[2], K[3], width, height};
+  // (+ 0.0: a principal point of -0 would give the projection's compare a -0)
+  k.cam = KaCam{K[0], K[1], K[2] + 0.0, K[3] + 0.0, width, height};
   k.cc = io->cauchy_c;
   k.st = st;
   k.nblk = 4 * sms;
   const size_t npix = (size_t)width * height;
   void* mem = nullptr;
-  const size_t bytes = sizeof(KaNormal) * npix + sizeof(double) * ((size_t)k.nblk * KA_NS + 64);
+  const size_t bytes = sizeof(KaNormal) * npix +
+                       sizeof(double) * ((size_t)k.nblk * KA_NS + KA_NS + width + height);
   VD_CU(cudaMallocAsync(&mem, bytes, st));
   k.n1 = (KaNormal*)mem;
   k.partial = (double*)(k.n1 + npix);
   k.sums = k.partial + (size_t)k.nblk * KA_NS;
-  k.Tdev = k.sums + 48;
+  k.rx = k.sums + KA_NS;
+  k.ry = k.rx + width;
   vd_status status = VD_OK;
   auto fail = [&](cudaError_t e) {
     vd_set_error(cudaGetErrorString(e));
@@ -293,10 +388,16 @@ extern "C" vd_status vd_ka_align(const float* depth1, const float* depth2, const
   for (int i = 0; i < 12; ++i) T[i] = io->pose[i];
   KaEval cur, cand;
   int it = 0;
+  k_ka_rays<<<(std::max(width, height) + KA_BLOCK - 1) / KA_BLOCK, KA_BLOCK, 0, st>>>(k.cam, k.rx,
+                                                                                      k.ry);
   k_ka_normals<<<(int)((npix + KA_BLOCK - 1) / KA_BLOCK), KA_BLOCK, 0, st>>>(depth1, k.cam, k.n1);
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = ka_eval(k, T, s, &cur);
+  if (e == cudaSuccess) e = ka_eval(k, T, s, true, &cur);
   double lam = KA_LAMBDA0;
+  // A refused step needs the energy only (half the time).  Refusals come in
+  // long runs or alternate with taken steps, so a step after three of them is
+  // evaluated by its energy first, and again in full if it is taken.
+  int refused = 0;
   while (e == cudaSuccess && it < io->max_iters && lam <= 1e10 && cur.n > 0) {
     ++it;
     double A[49], b[7], delta[7] = {0, 0, 0, 0, 0, 0, 0};
@@ -313,8 +414,12 @@ extern "C" vd_status vd_ka_align(const float* depth1, const float* depth2, const
     vd_se3_exp(delta, E6);
     vd_compose(E6, T, Tn);
     const double sn = io->fix_scale ? s : s * exp(delta[6]);
-    if ((e = ka_eval(k, Tn, sn, &cand)) != cudaSuccess) break;
-    if (cand.n > 0 && cand.E < cur.E) {
+    const bool full = refused < 3;
+    if ((e = ka_eval(k, Tn, sn, full, &cand)) != cudaSuccess) break;
+    const bool take = cand.n > 0 && cand.E < cur.E;
+    if (take && !full && (e = ka_eval(k, Tn, sn, true, &cand)) != cudaSuccess) break;
+    refused = take ? 0 : refused + 1;
+    if (take) {
       for (int i = 0; i < 12; ++i) T[i] = Tn[i];
       s = sn;
       cur = cand;
