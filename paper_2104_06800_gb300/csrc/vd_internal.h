@@ -177,6 +177,10 @@ int* vd_cnn_err_flag(vd_cnn* n);
 
 void vd_set_error(const char* msg);
 
+// Scratch of one call, in stream order; freed with cudaFreeAsync on the same
+// stream.
+cudaError_t vd_ws_alloc(void** p, size_t bytes, cudaStream_t s);
+
 // Return from a vd_status function on a CUDA error (recording its message).
 #define VD_CU(call)                                   \
   do {                                                \

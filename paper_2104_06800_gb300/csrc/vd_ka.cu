@@ -372,7 +372,7 @@ extern "C" vd_status vd_ka_align(const float* depth1, const float* depth2, const
   void* mem = nullptr;
   const size_t bytes = sizeof(KaNormal) * npix +
                        sizeof(double) * ((size_t)k.nblk * KA_NS + KA_NS + width + height);
-  VD_CU(cudaMallocAsync(&mem, bytes, st));
+  VD_CU(vd_ws_alloc(&mem, bytes, st));
   k.n1 = (KaNormal*)mem;
   k.partial = (double*)(k.n1 + npix);
   k.sums = k.partial + (size_t)k.nblk * KA_NS;

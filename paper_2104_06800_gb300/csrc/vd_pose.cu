@@ -1145,17 +1145,41 @@ cudaError_t launch_pose_frame(vd_ctx* c, uint32_t itcode, int t) {
 // ---------------------------------------------------------------------------
 // Standalone dense scoring on caller buffers (allocates its partial sums).
 // ---------------------------------------------------------------------------
-__global__ void k_poses_float(DevParams P, const double* __restrict__ poses, int m,
-                              float* __restrict__ out) {
+// K: the intrinsics (fx, fy, cx, cy) in device memory, or null: P's.
+__global__ void k_poses_float(DevParams P, const double* __restrict__ K,
+                              const double* __restrict__ poses, int m, float* __restrict__ out) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= m) return;
+  const double fx = K ? K[0] : P.fx_d, fy = K ? K[1] : P.fy_d;
+  const double cx = K ? K[2] : P.cx_d, cy = K ? K[3] : P.cy_d;
   const double* g = poses + 12 * r;
   float* o = out + 12 * r;
   for (int i = 0; i < 4; ++i) {
-    o[i < 3 ? i : 9] = (float)(P.fx_d * g[i] + P.cx_d * g[8 + i]);
-    o[i < 3 ? 3 + i : 10] = (float)(P.fy_d * g[4 + i] + P.cy_d * g[8 + i]);
+    o[i < 3 ? i : 9] = (float)(fx * g[i] + cx * g[8 + i]);
+    o[i < 3 ? 3 + i : 10] = (float)(fy * g[4 + i] + cy * g[8 + i]);
     o[i < 3 ? 6 + i : 11] = (float)g[8 + i];
   }
+}
+
+// Intrinsics of the standalone scoring: memory of the current device is read
+// by the kernel, in stream order; anything else is copied to K[4] first (a
+// blocking copy).
+static cudaError_t score_intrinsics(const double* in, double* K, const double** dev) {
+  *dev = nullptr;
+  int cur = 0;
+  cudaPointerAttributes a;
+  cudaError_t e = cudaGetDevice(&cur);
+  if (e != cudaSuccess) return e;
+  if (cudaPointerGetAttributes(&a, in) == cudaSuccess) {
+    if (a.type == cudaMemoryTypeDevice && a.device == cur) {
+      *dev = in;
+      K[0] = K[1] = K[2] = K[3] = 0.0;
+      return cudaSuccess;
+    }
+  } else {
+    cudaGetLastError();   // not an error of the call: the copy decides
+  }
+  return cudaMemcpy(K, in, 4 * sizeof(double), cudaMemcpyDefault);
 }
 
 // ---------------------------------------------------------------------------
@@ -1213,7 +1237,8 @@ extern "C" vd_status vd_score_poses_noalloc(const float* points, const float* ob
   int nblk = 0;
   cudaError_t e = noalloc_scratch(&scratch, &nblk);
   double K[4];
-  if (e == cudaSuccess) e = cudaMemcpy(K, intrinsics, sizeof K, cudaMemcpyDefault);
+  const double* Kdev = nullptr;
+  if (e == cudaSuccess) e = score_intrinsics(intrinsics, K, &Kdev);
   if (e != cudaSuccess) {
     vd_set_error(cudaGetErrorString(e));
     return VD_ERR_CUDA;
@@ -1226,7 +1251,7 @@ extern "C" vd_status vd_score_poses_noalloc(const float* points, const float* ob
   P.cgen = p0 * 2.0f * 3.14159265358979f / beta;
   float* rootsf = scratch;                                  // m x 12
   float* partial = scratch + 12 * VD_NOALLOC_MAX_POSES;     // m x nblk
-  k_poses_float<<<(m + 127) / 128, 128, 0, s>>>(P, poses, m, rootsf);
+  k_poses_float<<<(m + 127) / 128, 128, 0, s>>>(P, Kdev, poses, m, rootsf);
   const size_t smem = vd_score_smem(m, SCORE_THREADS);
   k_pose_score<SCORE_THREADS><<<dim3(nblk, (m + 31) / 32), SCORE_THREADS, smem, s>>>(
       P, (const float4*)points, (const float4*)obs, nullptr, n, rootsf, nullptr, m, partial);
@@ -1249,7 +1274,8 @@ extern "C" vd_status vd_score_poses(const float* points, const float* obs, int n
     return VD_ERR_ARG;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   double K[4];
-  if (cudaMemcpy(K, intrinsics, sizeof K, cudaMemcpyDefault) != cudaSuccess) {
+  const double* Kdev = nullptr;
+  if (score_intrinsics(intrinsics, K, &Kdev) != cudaSuccess) {
     vd_set_error(cudaGetErrorString(cudaGetLastError()));
     return VD_ERR_CUDA;
   }
@@ -1268,14 +1294,13 @@ extern "C" vd_status vd_score_poses(const float* points, const float* obs, int n
   const int nblk = 2 * std::max(sms, 1);
   float* rootsf = nullptr;
   float* partial = nullptr;
-  cudaError_t e = cudaMallocAsync(&rootsf, sizeof(float) * 12 * m, s);
-  if (e == cudaSuccess) e = cudaMallocAsync(&partial, sizeof(float) * (size_t)m * nblk, s);
+  cudaError_t e = vd_ws_alloc((void**)&rootsf, sizeof(float) * (size_t)m * (12 + nblk), s);
+  partial = rootsf + 12 * (size_t)m;
   if (e != cudaSuccess) {
-    if (rootsf) cudaFreeAsync(rootsf, s);
     vd_set_error(cudaGetErrorString(e));
     return VD_ERR_OOM;
   }
-  k_poses_float<<<(m + 127) / 128, 128, 0, s>>>(P, poses, m, rootsf);
+  k_poses_float<<<(m + 127) / 128, 128, 0, s>>>(P, Kdev, poses, m, rootsf);
   const size_t smem = vd_score_smem(m, SCORE_THREADS);
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(k_pose_score<SCORE_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1285,7 +1310,6 @@ extern "C" vd_status vd_score_poses(const float* points, const float* obs, int n
   launch_root_energy(partial, nblk, m, nullptr, energies, s);
   e = cudaGetLastError();
   cudaFreeAsync(rootsf, s);
-  cudaFreeAsync(partial, s);
   cudaError_t e2 = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) {
