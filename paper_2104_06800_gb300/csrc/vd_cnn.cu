@@ -364,6 +364,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap xmap, int Wimg, int Himg, int tile
   vd_tc_fence_before();
   __syncthreads();
   vd_tc_fence_after();
+  vd_pdl_begin();   // after the prologue, which touches no global memory
   const uint32_t dt = tmem_base;
   const uint32_t sB = (vd_smem_u32(smem) + 1023u) & ~1023u, sA = sB + S::A_OFF;
   const int my_tiles = blockIdx.x < n_tiles ? (n_tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
@@ -512,6 +513,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap xmap, int Wimg, int Himg, int tile
 __global__ void k_cnn_input(const float2* __restrict__ flow, int N, int Wimg, int HW, int C0,
                             const double* __restrict__ G1, float fx, float fy, float cx,
                             float cy, __nv_bfloat16* __restrict__ a0) {
+  vd_pdl_begin();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= HW) return;
   float geo[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -557,6 +559,7 @@ __global__ void k_cnn_input(const float2* __restrict__ flow, int N, int Wimg, in
 // ---------------------------------------------------------------------------
 __global__ void k_cnn_heads(const float* __restrict__ z, int HW, int N, float rho_min,
                             float rho_max, float* __restrict__ rho, float* __restrict__ q) {
+  vd_pdl_begin();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= HW) return;
   const float* v = z + (size_t)p * 16;
@@ -570,6 +573,7 @@ __global__ void k_cnn_loss(const float* __restrict__ z, int HW, int N,
                            const unsigned char* __restrict__ mask, float rho_min, float rho_max,
                            float w_q, const int* __restrict__ nmask,
                            __nv_bfloat16* __restrict__ dz, double* __restrict__ partial) {
+  vd_pdl_begin();
   __shared__ double s_l[256];
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   double l = 0.0;
@@ -622,6 +626,7 @@ __global__ void k_cnn_count(const unsigned char* __restrict__ mask, int HW, int*
 // a fixed order (strided per thread, then a tree), divided by the count.
 __global__ void k_cnn_sum(const double* __restrict__ partial, int n, const int* __restrict__ nmask,
                           double* __restrict__ out) {
+  vd_pdl_begin();
   __shared__ double s[1024];
   double v = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) v += partial[i];
@@ -734,6 +739,7 @@ k_wgrad_tc(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
   vd_tc_fence_before();
   __syncthreads();
   vd_tc_fence_after();
+  vd_pdl_begin();   // after the prologue, which touches no global memory
   const uint32_t dt = tmem_base;
   const uint32_t s0 = (vd_smem_u32(smem) + 1023u) & ~1023u;
   const int my_tiles = blockIdx.x < n_tiles ? (n_tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
@@ -898,6 +904,7 @@ __global__ void __launch_bounds__(256)
 k_cnn_wgrad_reduce(const float* __restrict__ partial, const float* __restrict__ partial_b,
                    int nblk, int stride, int nout, int stride_b, int cout,
                    float* __restrict__ gW, float* __restrict__ gb) {
+  vd_pdl_begin();
   __shared__ float s[8][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int o = blockIdx.x * 32 + lane;
@@ -1084,9 +1091,8 @@ static cudaError_t launch_conv(const __nv_bfloat16* X, int W, int H, const __nv_
   if (reinterpret_cast<uintptr_t>(Wt) & 15u) return cudaErrorInvalidValue;
   const int tiles_x = (W + CNN_TILE - 1) / CNN_TILE;
   const int n_tiles = tiles_x * ((H + R - 1) / R);
-  kern<<<min(n_tiles, slots), CNN_CONV_THREADS, S::SMEM, s>>>(map, W, H, tiles_x, n_tiles, Wt, b, out, mask,
-                                                 nout, err);
-  return cudaGetLastError();
+  return vd_launch(true, kern, min(n_tiles, slots), CNN_CONV_THREADS, S::SMEM, s, map, W, H, tiles_x,
+                   n_tiles, Wt, b, out, mask, nout, err);
 }
 
 // Forward pass of the whole network on flow [N][H][W][2] (device); keeps the
@@ -1148,14 +1154,13 @@ static cudaError_t launch_wgrad(vd_cnn* n, int l, const __nv_bfloat16* dz, int W
   if (e != cudaSuccess) return e;
   const int tiles_x = (W + CNN_TILE - 1) / CNN_TILE;
   const int n_tiles = tiles_x * ((H + WG_ROWS - 1) / WG_ROWS), nblk = min(n_tiles, slots);
-  kern<<<nblk, WG_THREADS, S::SMEM, s>>>(xmap, dmap, W, H, tiles_x, n_tiles, n->wg_partial,
-                                         n->wg_partial_b, n->err);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  e = vd_launch(true, kern, nblk, WG_THREADS, S::SMEM, s, xmap, dmap, W, H, tiles_x, n_tiles,
+                n->wg_partial, n->wg_partial_b, n->err);
+  if (e != cudaSuccess) return e;
   const int stride = COUT * 9 * CIN, nout = n->cout[l] * 9 * CIN;
-  k_cnn_wgrad_reduce<<<(nout + 31) / 32, 256, 0, s>>>(
-      n->wg_partial, n->wg_partial_b, nblk, stride, nout, COUT, n->cout[l],
-      n->grad + n->woff[l], n->grad + n->boff[l]);
-  return cudaGetLastError();
+  return vd_launch(true, k_cnn_wgrad_reduce, (nout + 31) / 32, 256, 0, s, n->wg_partial,
+                   n->wg_partial_b, nblk, stride, nout, COUT, n->cout[l], n->grad + n->woff[l],
+                   n->grad + n->boff[l]);
 }
 
 static cudaError_t cnn_backward(vd_cnn* n, int W, int H, cudaStream_t s) {
@@ -1409,9 +1414,8 @@ extern "C" vd_status vd_cnn_forward(vd_cnn* n, const float* flow, int width, int
   VD_CU(cnn_forward(n, flow, width, height, s, g));
   const int HW = width * height;
   if (rho_out || q_out) {
-    k_cnn_heads<<<(HW + 255) / 256, 256, 0, s>>>(n->zlast, HW, n->N, rho_min, rho_max, rho_out,
-                                                 q_out);
-    VD_CU(cudaGetLastError());
+    VD_CU(vd_launch(true, k_cnn_heads, (HW + 255) / 256, 256, 0, s, n->zlast, HW, n->N, rho_min,
+                    rho_max, rho_out, q_out));
   }
   return cnn_check_err(n, s);
 }
@@ -1433,10 +1437,10 @@ extern "C" vd_status vd_cnn_train_step(vd_cnn* n, const float* flow, int width, 
   const int nb = (HW + 255) / 256;
   VD_CU(cudaMemsetAsync(n->nmask, 0, sizeof(int), s));
   k_cnn_count<<<nb, 256, 0, s>>>(mask, HW, n->nmask);
-  k_cnn_loss<<<nb, 256, 0, s>>>(n->zlast, HW, n->N, rho_t, q_t, mask, rho_min, rho_max, w_q,
-                                n->nmask, n->g0, n->loss_partial);
-  k_cnn_sum<<<1, 1024, 0, s>>>(n->loss_partial, nb, n->nmask, n->loss);
   VD_CU(cudaGetLastError());
+  VD_CU(vd_launch(true, k_cnn_loss, nb, 256, 0, s, n->zlast, HW, n->N, rho_t, q_t, mask, rho_min,
+                  rho_max, w_q, n->nmask, n->g0, n->loss_partial));
+  VD_CU(vd_launch(true, k_cnn_sum, 1, 1024, 0, s, n->loss_partial, nb, n->nmask, n->loss));
   VD_CU(cnn_backward(n, width, height, s));
   if (update) {
     n->step += 1;

@@ -92,6 +92,7 @@ k_depth_sample(DevParams P, const float* __restrict__ posef, const float2* __res
                const float* __restrict__ prior_val, const float* __restrict__ prior_rho,
                const float* __restrict__ qhat, const float* __restrict__ pconf, uint32_t itcode,
                float s_pert, float* __restrict__ rho_star, float* __restrict__ e_star) {
+  vd_pdl_begin();
   __shared__ float sPose[12 * (VD_MAX_FLOWS + 1)];
   vd_load_pose_smem<NF>(sPose, posef);
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
@@ -247,6 +248,7 @@ k_depth_sample_q(DevParams P, const float* __restrict__ posef, const float2* __r
                  const float* __restrict__ qhat, const float* __restrict__ pconf,
                  uint32_t itcode, float s_pert, float* __restrict__ rho_star,
                  float* __restrict__ e_star) {
+  vd_pdl_begin();
   static_assert(NF >= 2, "the staged schedule needs a gathered flow term");
   constexpr int T1 = NF < VD_KQ_T1 ? NF : VD_KQ_T1;  // stage 1: flows [1, T1), stage 2: [T1, NF)
   __shared__ float sPose[12 * (VD_MAX_FLOWS + 1)];
@@ -440,6 +442,7 @@ k_propagate(DevParams P, const float* __restrict__ posef, const float2* __restri
             const float* __restrict__ qhat, const float* __restrict__ pconf,
             const float* __restrict__ rho_star, const float* __restrict__ e_star,
             float* __restrict__ rho_new, int direction, int restart, int s) {
+  vd_pdl_begin();
   extern __shared__ float sX[];                 // x, then in, of every pixel, then two lists of pixels
   __shared__ float sPose[12 * (VD_MAX_FLOWS + 1)];
   __shared__ int sStop[VD_PROP_MAX_THREADS];    // 4 d + kind of the first pixel that ends a try
@@ -565,6 +568,7 @@ k_hier_mix(DevParams P, const float* __restrict__ posef, const float2* __restric
            const float* __restrict__ rho_star, const float* __restrict__ e_star,
            const float* __restrict__ coarse, int s, float* __restrict__ rho_mid,
            float* __restrict__ e_mid) {
+  vd_pdl_begin();
   __shared__ float sPose[12 * (VD_MAX_FLOWS + 1)];
   vd_load_pose_smem<NF>(sPose, posef);
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
@@ -612,10 +616,11 @@ template <int WARPS>
 static cudaError_t launch_depth_sample_q(vd_ctx* c, uint32_t itcode, float s_pert, int nf) {
   const dim3 blk(32 * WARPS);
   const dim3 grd((c->W + 31) / 32, (c->H + WARPS - 1) / WARPS);
-  VD_DISPATCH_NF2(nf, (k_depth_sample_q<NF, WARPS><<<grd, blk, 0, c->stream>>>(
+  cudaError_t e = cudaSuccess;
+  VD_DISPATCH_NF2(nf, (e = vd_launch(vd_overlap(c), k_depth_sample_q<NF, WARPS>, grd, blk, 0, c->stream,
                           c->dp, c->posef, c->flow, c->rho, c->q, c->prior_val, c->prior_rho,
                           c->qhat, c->prior_conf, itcode, s_pert, c->rho_star, c->e_star)));
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_depth_sample(vd_ctx* c, uint32_t itcode, float s_pert, int nf) {
@@ -631,10 +636,11 @@ cudaError_t launch_depth_sample(vd_ctx* c, uint32_t itcode, float s_pert, int nf
 #endif
   const dim3 blk(VD_K1_BX, VD_K1_BY);
   const dim3 grd = pix_grid(c, blk);
-  VD_DISPATCH_NF(nf, (k_depth_sample<NF><<<grd, blk, 0, c->stream>>>(
+  cudaError_t e = cudaSuccess;
+  VD_DISPATCH_NF(nf, (e = vd_launch(vd_overlap(c), k_depth_sample<NF>, grd, blk, 0, c->stream,
                             c->dp, c->posef, c->flow, c->rho, c->q, c->prior_val, c->prior_rho,
                             c->qhat, c->prior_conf, itcode, s_pert, c->rho_star, c->e_star)));
-  return cudaGetLastError();
+  return e;
 }
 
 // Shared memory of the longest chain (16384 pixels), granted once per device
@@ -668,32 +674,34 @@ static size_t prop_smem(int L) { return (size_t)VD_PROP_ITEM_BYTES * L; }
 cudaError_t launch_depth_propagate(vd_ctx* c, int direction, int nf) {
   const bool rows = (direction & 1) == 0;
   const int nch = rows ? c->H : c->W, L = rows ? c->W : c->H;
+  cudaError_t e = cudaSuccess;
   if (!c->prm.hierarchical) {
-    VD_DISPATCH_NF(nf, (k_propagate<NF><<<nch, prop_threads(L), prop_smem(L), c->stream>>>(
+    VD_DISPATCH_NF(nf, (e = vd_launch(vd_overlap(c), k_propagate<NF>, nch, prop_threads(L), prop_smem(L),
+                              c->stream,
                               c->dp, c->posef, c->flow, c->q, c->prior_val, c->qhat, c->prior_conf,
                               c->rho_star, c->e_star, c->rho, direction, 0, 0)));
-    return cudaGetLastError();
+    return e;
   }
   const int s = c->prm.hier_scale;
   const int Wc = (c->W + s - 1) / s, Hc = (c->H + s - 1) / s;
   // global pass on the coarse grid: the same segmented exact chain walk
   const int Lc = rows ? Wc : Hc;
-  VD_DISPATCH_NF(nf, (k_propagate<NF><<<rows ? Hc : Wc, prop_threads(Lc), prop_smem(Lc), c->stream>>>(
+  VD_DISPATCH_NF(nf, (e = vd_launch(vd_overlap(c), k_propagate<NF>, rows ? Hc : Wc, prop_threads(Lc),
+                            prop_smem(Lc), c->stream,
                             c->dp, c->posef, c->flow, c->q, c->prior_val, c->qhat, c->prior_conf,
                             c->rho_star, c->e_star, c->coarse, direction, 0, s)));
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const dim3 blk(32, 4);
   const dim3 grd = pix_grid(c, blk);
-  VD_DISPATCH_NF(nf, (k_hier_mix<NF><<<grd, blk, 0, c->stream>>>(
+  VD_DISPATCH_NF(nf, (e = vd_launch(vd_overlap(c), k_hier_mix<NF>, grd, blk, 0, c->stream,
                             c->dp, c->posef, c->flow, c->q, c->prior_val, c->qhat, c->prior_conf,
                             c->rho_star, c->e_star, c->coarse, s, c->rho_mid, c->e_mid)));
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  VD_DISPATCH_NF(nf, (k_propagate<NF><<<nch, prop_threads(L), prop_smem(L), c->stream>>>(
+  VD_DISPATCH_NF(nf, (e = vd_launch(vd_overlap(c), k_propagate<NF>, nch, prop_threads(L), prop_smem(L),
+                              c->stream,
                             c->dp, c->posef, c->flow, c->q, c->prior_val, c->qhat, c->prior_conf,
                             c->rho_mid, c->e_mid, c->rho, direction, c->prm.hier_window, 0)));
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_eval_energy(vd_ctx* c, const float* rho_in, float* e_out) {

@@ -52,6 +52,14 @@ __device__ __forceinline__ long long vd_checked(int site, long long i, long long
 enum { VD_SITE_BILINEAR = 1, VD_SITE_P3P_TAPS = 2, VD_SITE_SCATTER = 3, VD_SITE_PICK = 4,
        VD_SITE_VC_CELL = 5, VD_SITE_CHAIN = 6 };
 
+// First statement of every kernel launched with vd_launch: waits for the
+// kernel before it (at once when the launch did not overlap it), then lets
+// the next one be placed.
+__device__ __forceinline__ void vd_pdl_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon et al., SC'11): ten rounds of two 32x32->64 bit
 // multiplies, mixing with the key, key advanced by the Weyl constants.

@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(128)
 k_emission(DevParams P, const float2* __restrict__ posed, const float2* __restrict__ flow,
            const float* __restrict__ rho, const float* __restrict__ prior_val,
            float* __restrict__ lam, float* __restrict__ qhat) {
+  vd_pdl_begin();
   __shared__ float2 sPose[12 * (VD_MAX_FLOWS + 1)];
   for (int i = threadIdx.x + threadIdx.y * blockDim.x; i < 12 * (NF + 1); i += blockDim.x * blockDim.y)
     sPose[i] = posed[i];
@@ -160,6 +161,7 @@ __device__ __forceinline__ VdM2 vd_m2_shfl_down(const VdM2& x, int off) {
 __global__ void __launch_bounds__(128)
 k_forward_backward_warp(DevParams P, const float* __restrict__ lam, float* __restrict__ q,
                         int direction) {
+  vd_pdl_begin();
   const bool rows = (direction & 1) == 0;
   const int nchains = rows ? P.H : P.W;
   const int L = rows ? P.W : P.H;
@@ -251,6 +253,7 @@ k_forward_backward_warp(DevParams P, const float* __restrict__ lam, float* __res
 __global__ void __launch_bounds__(256)
 k_forward_backward_staged(DevParams P, const float* __restrict__ lam, float* __restrict__ q,
                           int direction) {
+  vd_pdl_begin();
   extern __shared__ float fb_sm[];
   const bool rows = (direction & 1) == 0;
   const int nchains = rows ? P.H : P.W;
@@ -353,6 +356,7 @@ k_forward_backward_staged(DevParams P, const float* __restrict__ lam, float* __r
 // Eq. 6: C = (sum_t q_t + q_hat) / (N + 1) with a prior, sum_t q_t / N without.
 __global__ void k_confidence(DevParams P, const float* __restrict__ q,
                              const float* __restrict__ qhat, float* __restrict__ conf) {
+  vd_pdl_begin();
   const size_t npix = (size_t)P.W * P.H;
   const size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= npix) return;
@@ -371,9 +375,9 @@ __global__ void k_confidence(DevParams P, const float* __restrict__ q,
 cudaError_t launch_estep(vd_ctx* c, int direction) {
   const dim3 blk(32, 4);
   const dim3 grd((c->W + 31) / 32, (c->H + 3) / 4);
-  VD_DISPATCH_NF(c->N, (k_emission<NF><<<grd, blk, 0, c->stream>>>(
-                            c->dp, c->posed, c->flow, c->rho, c->prior_val, c->lam, c->qhat)));
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  VD_DISPATCH_NF(c->N, (e = vd_launch(vd_overlap(c), k_emission<NF>, grd, blk, 0, c->stream, c->dp,
+                                      c->posed, c->flow, c->rho, c->prior_val, c->lam, c->qhat)));
   if (e != cudaSuccess) return e;
   const bool rows = (direction & 1) == 0;
   const int nch = rows ? c->H : c->W, L = rows ? c->W : c->H;
@@ -384,18 +388,20 @@ cudaError_t launch_estep(vd_ctx* c, int direction) {
   int cb = rows ? 4 : 8;
   while (cb > 1 && cb * per_chain > 48 * 1024) cb >>= 1;
   if (cb * per_chain <= 48 * 1024) {
-    k_forward_backward_staged<<<dim3((nch + cb - 1) / cb, c->N), 32 * cb, cb * per_chain,
-                                c->stream>>>(c->dp, c->lam, c->q, direction);
+    // not overlapped, nor the confidence after it: its blocks need another
+    // split of the SM's memory into shared memory and cache than the kernels
+    // beside it, and an early launch then waits for the SMs to drain (a 160 x
+    // 120 E-step took 29 us overlapped, 20 not)
+    e = vd_launch(false, k_forward_backward_staged, dim3((nch + cb - 1) / cb, c->N), 32 * cb,
+                  cb * per_chain, c->stream, c->dp, c->lam, c->q, direction);
   } else {
     const int nwarps = nch * c->N;
-    k_forward_backward_warp<<<(nwarps + 3) / 4, 128, 0, c->stream>>>(c->dp, c->lam, c->q,
-                                                                      direction);
+    e = vd_launch(vd_overlap(c), k_forward_backward_warp, (nwarps + 3) / 4, 128, 0, c->stream, c->dp,
+                  c->lam, c->q, direction);
   }
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_confidence<<<(unsigned)((c->npix + 255) / 256), 256, 0, c->stream>>>(c->dp, c->q, c->qhat,
-                                                                         c->conf);
-  return cudaGetLastError();
+  return vd_launch(false, k_confidence, (unsigned)((c->npix + 255) / 256), 256, 0, c->stream,
+                   c->dp, c->q, c->qhat, c->conf);
 }
 
 VD_CHECK_ACCESSOR(estep)

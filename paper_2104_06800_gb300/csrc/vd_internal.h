@@ -190,6 +190,31 @@ cudaError_t vd_ws_alloc(void** p, size_t bytes, cudaStream_t s);
       return e_ == cudaErrorMemoryAllocation ? VD_ERR_OOM : VD_ERR_CUDA; \
     }                                                 \
   } while (0)
+// Launch of a kernel that begins with vd_pdl_begin (vd_device.cuh).  With
+// `overlap` the launch may be processed while the kernel before it on the
+// stream is running: its blocks are placed as soon as that kernel's have all
+// begun and there is room, and wait on the device for its end.  Every kernel
+// launched so waits before it touches memory, so a chain of them keeps the
+// stream's order.
+template <typename... K, typename... A>
+static inline cudaError_t vd_launch(bool overlap, void (*kern)(K...), dim3 grid, dim3 block,
+                                    size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<K>(args)...);
+}
+// Whether a context's launches overlap: not those of a batch, whose other
+// windows fill the SMs that a waiting block would hold.
+static inline bool vd_overlap(const vd_ctx* c) { return !c->batch_owned; }
+
 // stage profiling hooks (no-ops unless enabled); `n_launch` kernels are counted
 void vd_prof_begin(vd_ctx* c, int stage);
 void vd_prof_end(vd_ctx* c, int stage, int n_launch);

@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(SCAN_BLOCK)
 k_rigid_flags(DevParams P, const double* __restrict__ G, const float* __restrict__ posef,
               const float* __restrict__ rho, const float* __restrict__ q, int t,
               unsigned char* __restrict__ flags, int* __restrict__ blk_counts) {
+  vd_pdl_begin();
   const size_t npix = (size_t)P.W * P.H;
   const size_t j = (size_t)blockIdx.x * SCAN_BLOCK + threadIdx.x;
   int f = 0;
@@ -106,6 +107,7 @@ k_rigid_scatter(DevParams P, const float* __restrict__ posef, const float2* __re
                 const unsigned char* __restrict__ flags, const int* __restrict__ counts,
                 int* __restrict__ n_out, int* __restrict__ idx, float4* __restrict__ rpts,
                 float4* __restrict__ robs) {
+  vd_pdl_begin();
   __shared__ int warp_tot[SCAN_BLOCK / 32];
   __shared__ int warp_pre[SCAN_BLOCK / 32];
   const size_t npix = (size_t)P.W * P.H;
@@ -352,6 +354,7 @@ k_p3p_samples(DevParams P, const double* __restrict__ G, const float2* __restric
               const int* __restrict__ n_rigid, int t, uint32_t itcode, double* __restrict__ roots,
               int* __restrict__ root_count, float* __restrict__ rootsf,
               float* __restrict__ rootsr) {
+  vd_pdl_begin();
   const int g = blockIdx.x * VD_P3P_WARPS + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (g >= P.S) return;                       // whole warps leave together
@@ -556,6 +559,7 @@ __global__ void __launch_bounds__(THREADS)
 k_pose_score(DevParams P, const float4* __restrict__ rpts, const float4* __restrict__ robs,
              const int* __restrict__ n_ptr, int n_host, const float* __restrict__ rootsf,
              const int* __restrict__ root_count, int M, float* __restrict__ partial) {
+  vd_pdl_begin();
   extern __shared__ float smem[];
   constexpr int nwarp = THREADS / 32;
   constexpr int PASS = 32 * SCORE_PPT;
@@ -658,6 +662,7 @@ k_pose_score(DevParams P, const float4* __restrict__ rpts, const float4* __restr
 __global__ void k_root_energy(const float* __restrict__ partial, int nblk, int M,
                               const int* __restrict__ root_count, double* __restrict__ energy,
                               const int* __restrict__ n_ptr, unsigned long long* __restrict__ work) {
+  vd_pdl_begin();
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   const bool real = r < M && !(root_count && (r & 3) >= root_count[r >> 2]);
@@ -677,12 +682,12 @@ __global__ void k_root_energy(const float* __restrict__ partial, int nblk, int M
   if (lane == 0) energy[r] = s;
 }
 
-static inline cudaError_t launch_root_energy(const float* partial, int nblk, int M,
+static inline cudaError_t launch_root_energy(bool overlap, const float* partial, int nblk, int M,
                                              const int* root_count, double* energy,
                                              cudaStream_t s, const int* n_ptr = nullptr,
                                              unsigned long long* work = nullptr) {
-  k_root_energy<<<(M + 3) / 4, 128, 0, s>>>(partial, nblk, M, root_count, energy, n_ptr, work);
-  return cudaGetLastError();
+  return vd_launch(overlap, k_root_energy, (M + 3) / 4, 128, 0, s, partial, nblk, M, root_count,
+                   energy, n_ptr, work);
 }
 
 // ---------------------------------------------------------------------------
@@ -801,6 +806,7 @@ k_select_meanshift(DevParams P, const double* __restrict__ roots, const int* __r
                    float2* __restrict__ posed,
                    double* __restrict__ sample_pose, double* __restrict__ sample_energy,
                    int* __restrict__ degenerate) {
+  vd_pdl_begin();
   // one warp; lane l owns samples l, l + 32, ...
   __shared__ float sT[VD_MAX_SAMPLES][12];
   __shared__ unsigned char sValid[VD_MAX_SAMPLES];
@@ -1094,9 +1100,10 @@ cudaError_t launch_pose_score_only(vd_ctx* c) {
   // second dimension covers the root groups of 32 (those without a root exit)
   const int nblk = std::max(1, c->score_bps * c->num_sms / 2);
   const dim3 grid(nblk, (M + 31) / 32);
-#define VD_SCORE_LAUNCH(TH, FAST)                                                     \
-  k_pose_score<TH, FAST><<<grid, TH, vd_score_smem(M, TH), c->stream>>>(                   \
-      P, c->rpts, c->robs, c->n_rigid, 0, c->rootsf, c->root_count, M, c->partial)
+  cudaError_t e = cudaSuccess;
+#define VD_SCORE_LAUNCH(TH, FAST)                                                              \
+  e = vd_launch(vd_overlap(c), k_pose_score<TH, FAST>, grid, TH, vd_score_smem(M, TH), c->stream, \
+                P, c->rpts, c->robs, c->n_rigid, 0, c->rootsf, c->root_count, M, c->partial)
   if (c->score_threads == 512) {
     if (P.fast_beta2) VD_SCORE_LAUNCH(512, true);
     else VD_SCORE_LAUNCH(512, false);
@@ -1105,9 +1112,8 @@ cudaError_t launch_pose_score_only(vd_ctx* c) {
     else VD_SCORE_LAUNCH(256, false);
   }
 #undef VD_SCORE_LAUNCH
-  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_root_energy(c->partial, nblk, M, c->root_count, c->root_energy, c->stream,
+  return launch_root_energy(vd_overlap(c), c->partial, nblk, M, c->root_count, c->root_energy, c->stream,
                             c->n_rigid, c->score_work);
 }
 
@@ -1116,30 +1122,32 @@ cudaError_t launch_pose_frame(vd_ctx* c, uint32_t itcode, int t) {
   c->last_pose_t = t;
   c->samples_set |= 1u << (t - 1);
   const size_t f = (size_t)(t - 1) * VD_MAX_SAMPLES;   // this frame's sample slots
+  const bool ov = vd_overlap(c);
+  cudaError_t e = cudaSuccess;
   vd_prof_begin(c, VD_ST_RIGID);
-  k_rigid_flags<<<c->nblk_scan, SCAN_BLOCK, 0, c->stream>>>(P, c->G, c->posef, c->rho, c->q, t,
-                                                            c->flags, c->blk_counts);
-  k_rigid_scatter<<<c->nblk_scan, SCAN_BLOCK, 0, c->stream>>>(P, c->posef, c->flow, c->rho, c->q, t,
-                                                              c->flags, c->blk_counts,
-                                                              c->n_rigid, c->rigid_idx, c->rpts,
-                                                              c->robs);
+  e = vd_launch(ov, k_rigid_flags, c->nblk_scan, SCAN_BLOCK, 0, c->stream, P, c->G, c->posef, c->rho,
+                c->q, t, c->flags, c->blk_counts);
+  if (e != cudaSuccess) return e;
+  e = vd_launch(ov, k_rigid_scatter, c->nblk_scan, SCAN_BLOCK, 0, c->stream, P, c->posef, c->flow,
+                c->rho, c->q, t, c->flags, c->blk_counts, c->n_rigid, c->rigid_idx, c->rpts, c->robs);
+  if (e != cudaSuccess) return e;
   vd_prof_end(c, VD_ST_RIGID, 2);
   vd_prof_begin(c, VD_ST_P3P);
-  k_p3p_samples<<<(P.S + VD_P3P_WARPS - 1) / VD_P3P_WARPS, 32 * VD_P3P_WARPS, 0, c->stream>>>(
-      P, c->G, c->flow, c->rho, c->rigid_idx,
-                                            c->n_rigid, t, itcode, c->roots, c->root_count,
-                                            c->rootsf, c->rootsr);
+  e = vd_launch(ov, k_p3p_samples, (P.S + VD_P3P_WARPS - 1) / VD_P3P_WARPS, 32 * VD_P3P_WARPS, 0,
+                c->stream, P, c->G, c->flow, c->rho, c->rigid_idx, c->n_rigid, t, itcode, c->roots,
+                c->root_count, c->rootsf, c->rootsr);
+  if (e != cudaSuccess) return e;
   vd_prof_end(c, VD_ST_P3P, 1);
   vd_prof_begin(c, VD_ST_SCORE);
-  launch_pose_score_only(c);
+  e = launch_pose_score_only(c);
+  if (e != cudaSuccess) return e;
   vd_prof_end(c, VD_ST_SCORE, 2);
   vd_prof_begin(c, VD_ST_SELECT);
-  k_select_meanshift<<<1, 32, 0, c->stream>>>(P, c->roots, c->root_count, c->rootsr,
-                                               c->root_energy, t, c->G,
-                                               c->posef, c->posed, c->sample_pose + 12 * f,
-                                               c->sample_energy + f, c->degenerate);
+  e = vd_launch(ov, k_select_meanshift, 1, 32, 0, c->stream, P, c->roots, c->root_count, c->rootsr,
+                c->root_energy, t, c->G, c->posef, c->posed, c->sample_pose + 12 * f,
+                c->sample_energy + f, c->degenerate);
   vd_prof_end(c, VD_ST_SELECT, 1);
-  return cudaGetLastError();
+  return e;
 }
 
 // ---------------------------------------------------------------------------
@@ -1255,7 +1263,7 @@ extern "C" vd_status vd_score_poses_noalloc(const float* points, const float* ob
   const size_t smem = vd_score_smem(m, SCORE_THREADS);
   k_pose_score<SCORE_THREADS><<<dim3(nblk, (m + 31) / 32), SCORE_THREADS, smem, s>>>(
       P, (const float4*)points, (const float4*)obs, nullptr, n, rootsf, nullptr, m, partial);
-  launch_root_energy(partial, nblk, m, nullptr, energies, s);
+  launch_root_energy(true, partial, nblk, m, nullptr, energies, s);
   e = cudaGetLastError();
   cudaError_t e2 = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = e2;
@@ -1307,7 +1315,7 @@ extern "C" vd_status vd_score_poses(const float* points, const float* obs, int n
                          (int)smem);
   k_pose_score<SCORE_THREADS><<<dim3(nblk, (m + 31) / 32), SCORE_THREADS, smem, s>>>(
       P, (const float4*)points, (const float4*)obs, nullptr, n, rootsf, nullptr, m, partial);
-  launch_root_energy(partial, nblk, m, nullptr, energies, s);
+  launch_root_energy(true, partial, nblk, m, nullptr, energies, s);
   e = cudaGetLastError();
   cudaFreeAsync(rootsf, s);
   cudaError_t e2 = cudaStreamSynchronize(s);
