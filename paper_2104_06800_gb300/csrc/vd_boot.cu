@@ -87,7 +87,7 @@ __device__ __forceinline__ vd_df ep_shfl_xor(vd_df x, int o) {
 __global__ void __launch_bounds__(EP_THREADS, EP_MINB)
 k_ep_normal(DevParams P, const float2* __restrict__ flow, const double* __restrict__ Eprev,
             int weighted, float2* __restrict__ partial) {
-  vd_pdl_begin();
+  vd_pdl_begin(flow, Eprev);
   __shared__ vd_df sW[EP_THREADS / 32][45];
   vd_df acc[45];
 #pragma unroll
@@ -241,7 +241,7 @@ __device__ __forceinline__ void ep_inverse(const double* sM, double* sA, double*
 __global__ void __launch_bounds__(512)
 k_ep_solve(const float2* __restrict__ partial, int nblk, double* __restrict__ Mout,
            double* __restrict__ Eio, int warm) {
-  vd_pdl_begin();
+  vd_pdl_begin(partial);
   __shared__ double sM[45];
   __shared__ double sA[81];   // L (lower triangle)
   __shared__ double sRd[9];   // 1 / L_jj
@@ -354,7 +354,7 @@ k_ep_solve(const float2* __restrict__ partial, int nblk, double* __restrict__ Mo
 // U W^T V^T with translation +-U[:, 2] give the four candidate motions.
 __global__ void k_ep_decompose(const double* __restrict__ Ein, double* __restrict__ cand,
                                int* __restrict__ counts) {
-  vd_pdl_begin();
+  vd_pdl_begin(Ein);
   if (threadIdx.x != 0) return;
   double E[9];
   for (int i = 0; i < 9; ++i) E[i] = Ein[i];
@@ -412,7 +412,7 @@ __global__ void k_ep_decompose(const double* __restrict__ Ein, double* __restric
 __global__ void __launch_bounds__(EP_THREADS)
 k_ep_cheirality(DevParams P, const float2* __restrict__ flow, const double* __restrict__ cand,
                 int* __restrict__ counts) {
-  vd_pdl_begin();
+  vd_pdl_begin(flow, cand);
   __shared__ float sC[48];
   if (threadIdx.x < 48) sC[threadIdx.x] = (float)cand[threadIdx.x];
   __syncthreads();
@@ -456,7 +456,7 @@ k_ep_cheirality(DevParams P, const float2* __restrict__ flow, const double* __re
 __global__ void k_ep_finalize(DevParams P, const double* __restrict__ cand,
                               const int* __restrict__ counts, double* __restrict__ G,
                               float* __restrict__ posef, float2* __restrict__ posed) {
-  vd_pdl_begin();
+  vd_pdl_begin(cand, counts);
   if (threadIdx.x != 0) return;
   int best = 0;
   for (int k = 1; k < 4; ++k)

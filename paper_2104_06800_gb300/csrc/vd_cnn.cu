@@ -364,7 +364,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap xmap, int Wimg, int Himg, int tile
   vd_tc_fence_before();
   __syncthreads();
   vd_tc_fence_after();
-  vd_pdl_begin();   // after the prologue, which touches no global memory
+  vd_pdl_begin(Wt, bias, mask);   // after the prologue, which touches no global memory
   const uint32_t dt = tmem_base;
   const uint32_t sB = (vd_smem_u32(smem) + 1023u) & ~1023u, sA = sB + S::A_OFF;
   const int my_tiles = blockIdx.x < n_tiles ? (n_tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
@@ -513,7 +513,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap xmap, int Wimg, int Himg, int tile
 __global__ void k_cnn_input(const float2* __restrict__ flow, int N, int Wimg, int HW, int C0,
                             const double* __restrict__ G1, float fx, float fy, float cx,
                             float cy, __nv_bfloat16* __restrict__ a0) {
-  vd_pdl_begin();
+  vd_pdl_begin(flow, G1);
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= HW) return;
   float geo[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -559,7 +559,7 @@ __global__ void k_cnn_input(const float2* __restrict__ flow, int N, int Wimg, in
 // ---------------------------------------------------------------------------
 __global__ void k_cnn_heads(const float* __restrict__ z, int HW, int N, float rho_min,
                             float rho_max, float* __restrict__ rho, float* __restrict__ q) {
-  vd_pdl_begin();
+  vd_pdl_begin(z);
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= HW) return;
   const float* v = z + (size_t)p * 16;
@@ -573,7 +573,7 @@ __global__ void k_cnn_loss(const float* __restrict__ z, int HW, int N,
                            const unsigned char* __restrict__ mask, float rho_min, float rho_max,
                            float w_q, const int* __restrict__ nmask,
                            __nv_bfloat16* __restrict__ dz, double* __restrict__ partial) {
-  vd_pdl_begin();
+  vd_pdl_begin(z, rho_t, q_t, mask, nmask);
   __shared__ double s_l[256];
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   double l = 0.0;
@@ -626,7 +626,7 @@ __global__ void k_cnn_count(const unsigned char* __restrict__ mask, int HW, int*
 // a fixed order (strided per thread, then a tree), divided by the count.
 __global__ void k_cnn_sum(const double* __restrict__ partial, int n, const int* __restrict__ nmask,
                           double* __restrict__ out) {
-  vd_pdl_begin();
+  vd_pdl_begin(partial, nmask);
   __shared__ double s[1024];
   double v = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) v += partial[i];
@@ -904,7 +904,7 @@ __global__ void __launch_bounds__(256)
 k_cnn_wgrad_reduce(const float* __restrict__ partial, const float* __restrict__ partial_b,
                    int nblk, int stride, int nout, int stride_b, int cout,
                    float* __restrict__ gW, float* __restrict__ gb) {
-  vd_pdl_begin();
+  vd_pdl_begin(partial, partial_b);
   __shared__ float s[8][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int o = blockIdx.x * 32 + lane;

@@ -92,7 +92,7 @@ k_depth_sample(DevParams P, const float* __restrict__ posef, const float2* __res
                const float* __restrict__ prior_val, const float* __restrict__ prior_rho,
                const float* __restrict__ qhat, const float* __restrict__ pconf, uint32_t itcode,
                float s_pert, float* __restrict__ rho_star, float* __restrict__ e_star) {
-  vd_pdl_begin();
+  vd_pdl_begin(posef, flow, rho, q, prior_val, prior_rho, qhat, pconf);
   __shared__ float sPose[12 * (VD_MAX_FLOWS + 1)];
   vd_load_pose_smem<NF>(sPose, posef);
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
@@ -248,7 +248,7 @@ k_depth_sample_q(DevParams P, const float* __restrict__ posef, const float2* __r
                  const float* __restrict__ qhat, const float* __restrict__ pconf,
                  uint32_t itcode, float s_pert, float* __restrict__ rho_star,
                  float* __restrict__ e_star) {
-  vd_pdl_begin();
+  vd_pdl_begin(posef, flow, rho, q, prior_val, prior_rho, qhat, pconf);
   static_assert(NF >= 2, "the staged schedule needs a gathered flow term");
   constexpr int T1 = NF < VD_KQ_T1 ? NF : VD_KQ_T1;  // stage 1: flows [1, T1), stage 2: [T1, NF)
   __shared__ float sPose[12 * (VD_MAX_FLOWS + 1)];
@@ -442,7 +442,7 @@ k_propagate(DevParams P, const float* __restrict__ posef, const float2* __restri
             const float* __restrict__ qhat, const float* __restrict__ pconf,
             const float* __restrict__ rho_star, const float* __restrict__ e_star,
             float* __restrict__ rho_new, int direction, int restart, int s) {
-  vd_pdl_begin();
+  vd_pdl_begin(posef, flow, q, prior_val, qhat, pconf, rho_star, e_star);
   extern __shared__ float sX[];                 // x, then in, of every pixel, then two lists of pixels
   __shared__ float sPose[12 * (VD_MAX_FLOWS + 1)];
   __shared__ int sStop[VD_PROP_MAX_THREADS];    // 4 d + kind of the first pixel that ends a try
@@ -568,7 +568,7 @@ k_hier_mix(DevParams P, const float* __restrict__ posef, const float2* __restric
            const float* __restrict__ rho_star, const float* __restrict__ e_star,
            const float* __restrict__ coarse, int s, float* __restrict__ rho_mid,
            float* __restrict__ e_mid) {
-  vd_pdl_begin();
+  vd_pdl_begin(posef, flow, q, prior_val, qhat, pconf, rho_star, e_star, coarse);
   __shared__ float sPose[12 * (VD_MAX_FLOWS + 1)];
   vd_load_pose_smem<NF>(sPose, posef);
   const int u = blockIdx.x * blockDim.x + threadIdx.x;

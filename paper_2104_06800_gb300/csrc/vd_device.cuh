@@ -54,9 +54,24 @@ enum { VD_SITE_BILINEAR = 1, VD_SITE_P3P_TAPS = 2, VD_SITE_SCATTER = 3, VD_SITE_
 
 // First statement of every kernel launched with vd_launch: waits for the
 // kernel before it (at once when the launch did not overlap it), then lets
-// the next one be placed.
-__device__ __forceinline__ void vd_pdl_begin() {
+// the next one be placed.  An overlapped kernel exists while its predecessor
+// still writes, so its inputs are not read-only for its lifetime, which is
+// what `const __restrict__` tells the compiler: it may then load them by the
+// non-coherent path and before the wait.  Every such parameter is therefore
+// passed here, and its value comes out of the wait as one the compiler knows
+// nothing about.  Explicit __ldg stay for the flows, priors and rigidness: a
+// launch that does not overlap (the E-step's confidence, a copy) stands between
+// their writer and every reader.
+template <typename T>
+__device__ __forceinline__ void vd_pdl_hide(T& p) {
+  size_t a = __cvta_generic_to_global(p);
+  asm volatile("" : "+l"(a));
+  p = reinterpret_cast<T>(__cvta_global_to_generic(a));
+}
+template <typename... T>
+__device__ __forceinline__ void vd_pdl_begin(T&... inputs) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  (vd_pdl_hide(inputs), ...);
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(128)
 k_emission(DevParams P, const float2* __restrict__ posed, const float2* __restrict__ flow,
            const float* __restrict__ rho, const float* __restrict__ prior_val,
            float* __restrict__ lam, float* __restrict__ qhat) {
-  vd_pdl_begin();
+  vd_pdl_begin(posed, flow, rho, prior_val);
   __shared__ float2 sPose[12 * (VD_MAX_FLOWS + 1)];
   for (int i = threadIdx.x + threadIdx.y * blockDim.x; i < 12 * (NF + 1); i += blockDim.x * blockDim.y)
     sPose[i] = posed[i];
@@ -161,7 +161,7 @@ __device__ __forceinline__ VdM2 vd_m2_shfl_down(const VdM2& x, int off) {
 __global__ void __launch_bounds__(128)
 k_forward_backward_warp(DevParams P, const float* __restrict__ lam, float* __restrict__ q,
                         int direction) {
-  vd_pdl_begin();
+  vd_pdl_begin(lam);
   const bool rows = (direction & 1) == 0;
   const int nchains = rows ? P.H : P.W;
   const int L = rows ? P.W : P.H;
@@ -253,7 +253,7 @@ k_forward_backward_warp(DevParams P, const float* __restrict__ lam, float* __res
 __global__ void __launch_bounds__(256)
 k_forward_backward_staged(DevParams P, const float* __restrict__ lam, float* __restrict__ q,
                           int direction) {
-  vd_pdl_begin();
+  vd_pdl_begin(lam);
   extern __shared__ float fb_sm[];
   const bool rows = (direction & 1) == 0;
   const int nchains = rows ? P.H : P.W;
@@ -356,7 +356,7 @@ k_forward_backward_staged(DevParams P, const float* __restrict__ lam, float* __r
 // Eq. 6: C = (sum_t q_t + q_hat) / (N + 1) with a prior, sum_t q_t / N without.
 __global__ void k_confidence(DevParams P, const float* __restrict__ q,
                              const float* __restrict__ qhat, float* __restrict__ conf) {
-  vd_pdl_begin();
+  vd_pdl_begin(q, qhat);
   const size_t npix = (size_t)P.W * P.H;
   const size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= npix) return;

@@ -209,7 +209,10 @@ static inline cudaError_t vd_launch(bool overlap, void (*kern)(K...), dim3 grid,
   cfg.stream = s;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<K>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<K>(args)...);
+  // the error is returned and left nowhere else: the caller's next CUDA call
+  // on this thread does not meet it again
+  return e == cudaSuccess ? cudaGetLastError() : (cudaGetLastError(), e);
 }
 // Whether a context's launches overlap: not those of a batch, whose other
 // windows fill the SMs that a waiting block would hold.

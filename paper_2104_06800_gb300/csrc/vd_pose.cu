@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(SCAN_BLOCK)
 k_rigid_flags(DevParams P, const double* __restrict__ G, const float* __restrict__ posef,
               const float* __restrict__ rho, const float* __restrict__ q, int t,
               unsigned char* __restrict__ flags, int* __restrict__ blk_counts) {
-  vd_pdl_begin();
+  vd_pdl_begin(G, posef, rho, q);
   const size_t npix = (size_t)P.W * P.H;
   const size_t j = (size_t)blockIdx.x * SCAN_BLOCK + threadIdx.x;
   int f = 0;
@@ -107,7 +107,7 @@ k_rigid_scatter(DevParams P, const float* __restrict__ posef, const float2* __re
                 const unsigned char* __restrict__ flags, const int* __restrict__ counts,
                 int* __restrict__ n_out, int* __restrict__ idx, float4* __restrict__ rpts,
                 float4* __restrict__ robs) {
-  vd_pdl_begin();
+  vd_pdl_begin(posef, flow, rho, q, flags, counts);
   __shared__ int warp_tot[SCAN_BLOCK / 32];
   __shared__ int warp_pre[SCAN_BLOCK / 32];
   const size_t npix = (size_t)P.W * P.H;
@@ -354,7 +354,7 @@ k_p3p_samples(DevParams P, const double* __restrict__ G, const float2* __restric
               const int* __restrict__ n_rigid, int t, uint32_t itcode, double* __restrict__ roots,
               int* __restrict__ root_count, float* __restrict__ rootsf,
               float* __restrict__ rootsr) {
-  vd_pdl_begin();
+  vd_pdl_begin(G, flow, rho, idx, n_rigid);
   const int g = blockIdx.x * VD_P3P_WARPS + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (g >= P.S) return;                       // whole warps leave together
@@ -559,7 +559,7 @@ __global__ void __launch_bounds__(THREADS)
 k_pose_score(DevParams P, const float4* __restrict__ rpts, const float4* __restrict__ robs,
              const int* __restrict__ n_ptr, int n_host, const float* __restrict__ rootsf,
              const int* __restrict__ root_count, int M, float* __restrict__ partial) {
-  vd_pdl_begin();
+  vd_pdl_begin(rpts, robs, n_ptr, rootsf, root_count);
   extern __shared__ float smem[];
   constexpr int nwarp = THREADS / 32;
   constexpr int PASS = 32 * SCORE_PPT;
@@ -662,7 +662,7 @@ k_pose_score(DevParams P, const float4* __restrict__ rpts, const float4* __restr
 __global__ void k_root_energy(const float* __restrict__ partial, int nblk, int M,
                               const int* __restrict__ root_count, double* __restrict__ energy,
                               const int* __restrict__ n_ptr, unsigned long long* __restrict__ work) {
-  vd_pdl_begin();
+  vd_pdl_begin(partial, root_count, n_ptr);
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   const bool real = r < M && !(root_count && (r & 3) >= root_count[r >> 2]);
@@ -806,7 +806,7 @@ k_select_meanshift(DevParams P, const double* __restrict__ roots, const int* __r
                    float2* __restrict__ posed,
                    double* __restrict__ sample_pose, double* __restrict__ sample_energy,
                    int* __restrict__ degenerate) {
-  vd_pdl_begin();
+  vd_pdl_begin(roots, root_count, roots_r, root_energy);
   // one warp; lane l owns samples l, l + 32, ...
   __shared__ float sT[VD_MAX_SAMPLES][12];
   __shared__ unsigned char sValid[VD_MAX_SAMPLES];
@@ -1263,8 +1263,7 @@ extern "C" vd_status vd_score_poses_noalloc(const float* points, const float* ob
   const size_t smem = vd_score_smem(m, SCORE_THREADS);
   k_pose_score<SCORE_THREADS><<<dim3(nblk, (m + 31) / 32), SCORE_THREADS, smem, s>>>(
       P, (const float4*)points, (const float4*)obs, nullptr, n, rootsf, nullptr, m, partial);
-  launch_root_energy(true, partial, nblk, m, nullptr, energies, s);
-  e = cudaGetLastError();
+  e = launch_root_energy(true, partial, nblk, m, nullptr, energies, s);
   cudaError_t e2 = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) {
@@ -1315,8 +1314,7 @@ extern "C" vd_status vd_score_poses(const float* points, const float* obs, int n
                          (int)smem);
   k_pose_score<SCORE_THREADS><<<dim3(nblk, (m + 31) / 32), SCORE_THREADS, smem, s>>>(
       P, (const float4*)points, (const float4*)obs, nullptr, n, rootsf, nullptr, m, partial);
-  launch_root_energy(true, partial, nblk, m, nullptr, energies, s);
-  e = cudaGetLastError();
+  e = launch_root_energy(true, partial, nblk, m, nullptr, energies, s);
   cudaFreeAsync(rootsf, s);
   cudaError_t e2 = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = e2;
