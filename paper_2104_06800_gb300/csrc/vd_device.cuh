@@ -121,6 +121,62 @@ __device__ __forceinline__ float vd_clamp(float c, float lo, float hi) {
 // uniform.  Returned in log2 units (multiply by ln 2).  Also returns
 // y = P0 / p1 (the outlier-to-rigid likelihood ratio) for the E-step.
 // ---------------------------------------------------------------------------
+// 1 / x and log2 x of the special-function unit for x in float32's normal
+// range: __fdividef and __log2f less the instructions that rescale subnormals
+// (the same bits; three to four instructions fewer per call).
+__device__ __forceinline__ float vd_rcp(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float vd_ex2(float x) {   // 0 below 2^-126
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float vd_lg2(float x) {
+  float r;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// Two float32 values in one 64-bit register pair.  The packed instructions
+// round each half exactly as the scalar ones do, and cost one issue slot for
+// both: what the issue-bound kernels (depth sampling, pose scoring) use them
+// for.
+typedef unsigned long long vd_f2;
+__device__ __forceinline__ vd_f2 vd_pack(float lo, float hi) {
+  vd_f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void vd_unpack(vd_f2 a, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
+}
+__device__ __forceinline__ vd_f2 vd_fma2(vd_f2 a, vd_f2 b, vd_f2 c) {
+  vd_f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ vd_f2 vd_mul2(vd_f2 a, vd_f2 b) {
+  vd_f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ vd_f2 vd_add2(vd_f2 a, vd_f2 b) {
+  vd_f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ vd_f2 vd_sub2(vd_f2 a, vd_f2 b) {
+  vd_f2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+__device__ __forceinline__ float vd_lo(vd_f2 a) { return __uint_as_float((unsigned)a); }
+__device__ __forceinline__ float vd_hi(vd_f2 a) { return __uint_as_float((unsigned)(a >> 32)); }
+
 __device__ __forceinline__ float vd_ratio_general(const DevParams& P, float r2, float alpha) {
   float r = sqrtf(r2);
   if (P.beta != 2.0f) r = fmaxf(r, VD_R_FLOOR);

@@ -466,6 +466,15 @@ k_p3p_samples(DevParams P, const double* __restrict__ G, const float2* __restric
 // root in every lane; a butterfly reduce-scatter (31 shuffles) then leaves
 // lane L holding the warp's sum of root 32 g + L.  Warp sums are added in
 // fixed order, so the result does not depend on scheduling.
+//
+// Bound: issue slots (31 warp instructions a pixel and root with scalar
+// arithmetic, 21 of them float32).  Two pixels share one packed instruction
+// wherever their arithmetic is the same, with the same rounding, and the
+// root's entries lie twice in shared memory for it; the reciprocal and the
+// logarithm skip the rescaling of subnormals that cannot occur.  Same results;
+// a 1216 x 368 window of 6 flows and 8 iterations 12.28 -> 11.78 ms, a pose
+// step of 5 frames of 640 x 480 556 -> 537 us, 300001 points of their own
+// scale under 256 poses 257 -> 226 us a call (with its synchronisation).
 // ---------------------------------------------------------------------------
 #ifndef VD_SCORE_PPT
 #define VD_SCORE_PPT 4
@@ -473,42 +482,135 @@ k_p3p_samples(DevParams P, const double* __restrict__ G, const float2* __restric
 #undef SCORE_PPT
 #define SCORE_PPT VD_SCORE_PPT
 
-// One pixel's term under one root in log2 units (the caller scales by ln 2),
-// without branches.  FAST: beta = 2 and alpha1 = 0 (closed form; obs.z
-// unused) with one MUFU log2: log2(1 + y) below y = 2^24, log2 y = log2 c0 +
-// 2 log2 s above (equal to float32 precision there, and no overflow), the
-// series of ln(1 + y) below y = 1/32.  A point behind the camera gives the
-// constant term (its projection uses a denominator of 1 and is discarded).
-template <bool FAST>
-__device__ __forceinline__ float vd_score_term2(const DevParams& P, const float* Mr, float4 pt,
-                                                float4 ob) {
-  const float hx = fmaf(Mr[0], pt.x, fmaf(Mr[1], pt.y, fmaf(Mr[2], pt.z, Mr[9])));
-  const float hy = fmaf(Mr[3], pt.x, fmaf(Mr[4], pt.y, fmaf(Mr[5], pt.z, Mr[10])));
-  const float hz = fmaf(Mr[6], pt.x, fmaf(Mr[7], pt.y, fmaf(Mr[8], pt.z, Mr[11])));
-  const bool front = hz > VD_Z_EPS;
-  const float iz = __fdividef(1.0f, front ? hz : 1.0f);
-  const float dx = fmaf(-hx, iz, ob.x), dy = fmaf(-hy, iz, ob.y);
-  const float r2 = fmaf(dx, dx, dy * dy);
-  float l2;
-  if (FAST) {
-    const float sq = fmaf(r2, P.inv_a2, 1.0f);
-    const float y = P.c0 * sq * sq;
-    const bool mid = y < 16777216.0f;
-    const float L = __log2f(mid ? 1.0f + y : sq);
-    const float big = mid ? L : fmaf(2.0f, L, P.log2c0);
-    // log2(1 + y) = y (1 - y/2 + y^2/3 - y^3/4 + y^4/5) / ln 2 (below 1/32)
-    const float ser = y * fmaf(y, fmaf(y, fmaf(y, fmaf(y, 0.28853901f, -0.36067376f),
-                                                0.48089835f), -0.72134752f), 1.44269504f);
-    l2 = y < 0.03125f ? ser : big;
-  } else {
-    l2 = vd_l2_general(P, r2, ob.z);
+// What a pixel's term needs, by the residual density: beta = 2 with one scale
+// for all pixels (the closed form with the launch's constants), beta = 2 with
+// a scale per pixel (its reciprocal and P0 pi alpha^2 are formed once per pixel
+// and pass, for 32 roots), and any beta.
+enum { VD_SCORE_UNIFORM = 0, VD_SCORE_SCALED = 1, VD_SCORE_GENERAL = 2 };
+
+// Two pixels side by side: point, observation and scale.
+template <int MODE>
+struct VdScorePair {
+  vd_f2 X, Y, Z, ox, oy;
+  vd_f2 nal, ial, c;          // scaled: -alpha, 1 / alpha, P0 pi alpha^2
+  float a0, a1;               // general: alpha
+  float w0, w1;
+  __device__ __forceinline__ void load(const DevParams& P, float4 p0, float4 o0, float4 p1,
+                                       float4 o1) {
+    X = vd_pack(p0.x, p1.x);
+    Y = vd_pack(p0.y, p1.y);
+    Z = vd_pack(p0.z, p1.z);
+    w0 = p0.w;
+    w1 = p1.w;
+    ox = vd_pack(o0.x, o1.x);
+    oy = vd_pack(o0.y, o1.y);
+    a0 = o0.z;
+    a1 = o1.z;
+    nal = vd_pack(-a0, -a1);
+    ial = vd_pack(__frcp_rn(a0), __frcp_rn(a1));
+    c = vd_pack(P.cgen * a0 * a0, P.cgen * a1 * a1);
   }
-  return front ? l2 : VD_L_BEHIND / VD_LN2;
+};
+
+// The scaled terms' quotient s = r / alpha comes from the rounded reciprocal
+// and the remainder of the first quotient (Markstein's correction): the bits
+// of a division, but for exact quotients within 2^-23 of a last place of a
+// rounding boundary, in three packed operations.  2 - beta is 0, so the
+// general form's second exponential is 1 (and NaN at log2 s = +-inf, as
+// 0 * inf is).
+__device__ __forceinline__ void vd_score_scaled(const DevParams& P, vd_f2 r2, vd_f2 nal, vd_f2 ial,
+                                                vd_f2 c, float a0, float a1, float* l0, float* l1) {
+  const vd_f2 one = vd_pack(1.0f, 1.0f);
+  const float ra = vd_lo(r2), rb = vd_hi(r2);
+  const vd_f2 r = vd_pack(sqrtf(ra), sqrtf(rb));
+  const vd_f2 q = vd_mul2(r, ial);
+  const vd_f2 s = vd_fma2(vd_fma2(q, nal, r), ial, q);
+  const vd_f2 ls = vd_pack(__log2f(vd_lo(s)), __log2f(vd_hi(s)));
+  const vd_f2 e = vd_add2(ls, ls);
+  const vd_f2 u = vd_add2(one, vd_pack(vd_ex2(vd_lo(e)), vd_ex2(vd_hi(e))));
+  const vd_f2 s2b = vd_fma2(ls, 0, one);
+  const vd_f2 y = vd_mul2(vd_mul2(vd_mul2(c, s2b), u), u);
+  const float y0 = vd_lo(y), y1 = vd_hi(y);
+  if (!(y0 < 1e30f && y1 < 1e30f)) {            // overflow or NaN: the general form
+    *l0 = vd_l2_general(P, ra, a0);
+    *l1 = vd_l2_general(P, rb, a1);
+    return;
+  }
+  const vd_f2 v = vd_add2(one, y);
+  // vd_ell2
+  vd_f2 t = vd_fma2(y, vd_pack(0.2f, 0.2f), vd_pack(-0.25f, -0.25f));
+  t = vd_fma2(y, t, vd_pack(0.33333334f, 0.33333334f));
+  t = vd_fma2(y, t, vd_pack(-0.5f, -0.5f));
+  t = vd_fma2(y, t, one);
+  t = vd_mul2(vd_mul2(y, t), vd_pack(1.44269504f, 1.44269504f));
+  *l0 = y0 < 0.03125f ? vd_lo(t) : vd_lg2(vd_lo(v));
+  *l1 = y1 < 0.03125f ? vd_hi(t) : vd_lg2(vd_hi(v));
+}
+
+// The terms of two pixels under one root in log2 units (the caller scales by
+// ln 2).  Uniform: without branches, one MUFU log2 each, log2(1 + y) below
+// y = 2^24, log2 y = log2 c0 + 2 log2 s above (equal to float32 precision
+// there, and no overflow), the series of ln(1 + y) below y = 1/32.  A point
+// behind the camera gives the constant term (its projection uses a
+// denominator of 1 and is discarded).  Mr: the root's 12 entries, each twice,
+// those of the image rows x and y negated (so that the residual is one packed
+// multiply-add).
+template <int MODE>
+__device__ __forceinline__ void vd_score_pair(const DevParams& P, const float4* Mr,
+                                              const VdScorePair<MODE>& p, float* l0, float* l1) {
+  vd_f2 m[12];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const float4 v = Mr[i];
+    m[2 * i] = vd_pack(v.x, v.y);
+    m[2 * i + 1] = vd_pack(v.z, v.w);
+  }
+  const vd_f2 hx = vd_fma2(m[0], p.X, vd_fma2(m[1], p.Y, vd_fma2(m[2], p.Z, m[9])));
+  const vd_f2 hy = vd_fma2(m[3], p.X, vd_fma2(m[4], p.Y, vd_fma2(m[5], p.Z, m[10])));
+  const vd_f2 hz = vd_fma2(m[6], p.X, vd_fma2(m[7], p.Y, vd_fma2(m[8], p.Z, m[11])));
+  float z0, z1;
+  vd_unpack(hz, z0, z1);
+  const bool f0 = z0 > VD_Z_EPS, f1 = z1 > VD_Z_EPS;
+  const vd_f2 iz = vd_pack(vd_rcp(f0 ? z0 : 1.0f), vd_rcp(f1 ? z1 : 1.0f));
+  const vd_f2 dx = vd_fma2(hx, iz, p.ox), dy = vd_fma2(hy, iz, p.oy);
+  const vd_f2 r2 = vd_fma2(dx, dx, vd_mul2(dy, dy));
+  float a, b;
+  if (MODE == VD_SCORE_GENERAL) {
+    float ra, rb;
+    vd_unpack(r2, ra, rb);
+    a = vd_l2_general(P, ra, p.a0);
+    b = vd_l2_general(P, rb, p.a1);
+  } else if (MODE == VD_SCORE_SCALED) {
+    vd_score_scaled(P, r2, p.nal, p.ial, p.c, p.a0, p.a1, &a, &b);
+  } else {
+    const vd_f2 one = vd_pack(1.0f, 1.0f);
+    const vd_f2 sq = vd_fma2(r2, vd_pack(P.inv_a2, P.inv_a2), one);
+    const vd_f2 y = vd_mul2(vd_mul2(vd_pack(P.c0, P.c0), sq), sq);
+    float y0, y1, u0, u1, s0, s1;
+    vd_unpack(y, y0, y1);
+    vd_unpack(vd_add2(one, y), u0, u1);
+    vd_unpack(sq, s0, s1);
+    const bool mid0 = y0 < 16777216.0f, mid1 = y1 < 16777216.0f;
+    const float L0 = vd_lg2(mid0 ? u0 : s0), L1 = vd_lg2(mid1 ? u1 : s1);
+    const float big0 = mid0 ? L0 : fmaf(2.0f, L0, P.log2c0);
+    const float big1 = mid1 ? L1 : fmaf(2.0f, L1, P.log2c0);
+    // log2(1 + y) = y (1 - y/2 + y^2/3 - y^3/4 + y^4/5) / ln 2 (below 1/32)
+    vd_f2 t = vd_fma2(y, vd_pack(0.28853901f, 0.28853901f), vd_pack(-0.36067376f, -0.36067376f));
+    t = vd_fma2(y, t, vd_pack(0.48089835f, 0.48089835f));
+    t = vd_fma2(y, t, vd_pack(-0.72134752f, -0.72134752f));
+    t = vd_fma2(y, t, vd_pack(1.44269504f, 1.44269504f));
+    float e0, e1;
+    vd_unpack(vd_mul2(y, t), e0, e1);
+    a = y0 < 0.03125f ? e0 : big0;
+    b = y1 < 0.03125f ? e1 : big1;
+  }
+  *l0 = f0 ? a : VD_L_BEHIND / VD_LN2;
+  *l1 = f1 ? b : VD_L_BEHIND / VD_LN2;
 }
 
 // Dynamic shared memory of k_pose_score<THREADS> for M roots.
 static inline size_t vd_score_smem(int M, int threads) {
-  return sizeof(float) * (size_t)32 * (12 + threads / 32) + sizeof(int) * (size_t)(M + 1);
+  return sizeof(float) * (size_t)32 * (24 + threads / 32) + sizeof(int) * (size_t)(M + 1);
 }
 
 // acc[0..7] of every lane -> lanes with L % 8 == k return the warp's sum of
@@ -554,17 +656,18 @@ __device__ __forceinline__ float vd_reduce_scatter32(float* acc, int lane) {
 // root over its pixels, then a reduce-scatter gives lane k < 8 the warp's
 // sum of root k.  Warp sums are added in fixed order, so the result does
 // not depend on scheduling.
-template <int THREADS, bool FAST = false>
+template <int THREADS, int MODE>
 __global__ void __launch_bounds__(THREADS)
 k_pose_score(DevParams P, const float4* __restrict__ rpts, const float4* __restrict__ robs,
              const int* __restrict__ n_ptr, int n_host, const float* __restrict__ rootsf,
              const int* __restrict__ root_count, int M, float* __restrict__ partial) {
   vd_pdl_begin(rpts, robs, n_ptr, rootsf, root_count);
-  extern __shared__ float smem[];
+  extern __shared__ __align__(16) float smem[];
   constexpr int nwarp = THREADS / 32;
   constexpr int PASS = 32 * SCORE_PPT;
-  float* sRoot = smem;                       // 32 * 12: this group's roots
-  float* sAcc = smem + 32 * 12;              // nwarp * 32
+  static_assert(SCORE_PPT % 2 == 0, "pixels are scored in pairs");
+  float* sRoot = smem;                       // 32 * 24: this group's roots (vd_score_pair)
+  float* sAcc = smem + 32 * 24;              // nwarp * 32
   int* sList = (int*)(sAcc + nwarp * 32);    // the real roots, in index order
   int* sNum = sList + M;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -607,8 +710,12 @@ k_pose_score(DevParams P, const float4* __restrict__ rpts, const float4* __restr
   const int g0 = 32 * blockIdx.y;
   if (g0 >= nroot) return;                   // whole block: no root in this group
   const int ng = min(32, nroot - g0);
-  for (int i = threadIdx.x; i < 12 * ng; i += THREADS)
-    sRoot[i] = rootsf[12 * sList[g0 + i / 12] + i % 12];
+  for (int i = threadIdx.x; i < 12 * ng; i += THREADS) {
+    const int e = i % 12;
+    const float m = rootsf[12 * sList[g0 + i / 12] + e];
+    const float v = e < 6 || e == 9 || e == 10 ? -m : m;   // rows x and y of K [R | tau]
+    reinterpret_cast<float2*>(sRoot)[i] = make_float2(v, v);
+  }
   __syncthreads();
   // contiguous pixel-block ranges of whole passes; passes go to the warps in turn
   const int per = ((n + gridDim.x - 1) / gridDim.x + PASS - 1) / PASS * PASS;
@@ -616,17 +723,14 @@ k_pose_score(DevParams P, const float4* __restrict__ rpts, const float4* __restr
   const int end = min(n, beg + per);
   float* wAcc = sAcc + wid * 32;             // this warp's sum per root of the group
   for (int base = beg + wid * PASS; base < end; base += nwarp * PASS) {
-    float4 pt[SCORE_PPT], ob[SCORE_PPT];
+    VdScorePair<MODE> px[SCORE_PPT / 2];
+    const float4 none = make_float4(0.f, 0.f, 1.f, 0.f);   // weight 0, scale 1
 #pragma unroll
-    for (int k = 0; k < SCORE_PPT; ++k) {
-      const int i = base + 32 * k + lane;
-      if (i < end) {
-        pt[k] = rpts[i];
-        ob[k] = robs[i];
-      } else {
-        pt[k] = make_float4(0.f, 0.f, 1.f, 0.f);   // weight 0
-        ob[k] = make_float4(0.f, 0.f, 1.f, 0.f);
-      }
+    for (int k = 0; k < SCORE_PPT / 2; ++k) {
+      const int i = base + 64 * k + lane;
+      const bool in0 = i < end, in1 = i + 32 < end;
+      px[k].load(P, in0 ? rpts[i] : none, in0 ? robs[i] : none, in1 ? rpts[i + 32] : none,
+                 in1 ? robs[i + 32] : none);
     }
 #pragma unroll 1
     for (int r0 = 0; r0 < ng; r0 += 8) {
@@ -635,10 +739,13 @@ k_pose_score(DevParams P, const float4* __restrict__ rpts, const float4* __restr
       for (int k = 0; k < 8; ++k) {
         acc[k] = 0.0f;
         if (r0 + k < ng) {                    // warp-uniform
-          const float* Mr = sRoot + 12 * (r0 + k);
+          const float4* Mr = reinterpret_cast<const float4*>(sRoot) + 6 * (r0 + k);
 #pragma unroll
-          for (int q = 0; q < SCORE_PPT; ++q)
-            acc[k] = fmaf(pt[q].w, vd_score_term2<FAST>(P, Mr, pt[q], ob[q]), acc[k]);
+          for (int q = 0; q < SCORE_PPT / 2; ++q) {
+            float l0, l1;
+            vd_score_pair<MODE>(P, Mr, px[q], &l0, &l1);
+            acc[k] = fmaf(px[q].w1, l1, fmaf(px[q].w0, l0, acc[k]));
+          }
         }
       }
       const float v = vd_reduce_scatter8(acc, lane);
@@ -1084,10 +1191,12 @@ cudaError_t vd_pose_prepare(void) {
   const int M = 4 * VD_MAX_SAMPLES;
   const int s256 = (int)vd_score_smem(M, 256), s512 = (int)vd_score_smem(M, 512);
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(k_pose_score<256, false>, a, s256);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pose_score<256, true>, a, s256);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pose_score<512, false>, a, s512);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pose_score<512, true>, a, s512);
+  cudaError_t e = cudaFuncSetAttribute(k_pose_score<256, VD_SCORE_GENERAL>, a, s256);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pose_score<256, VD_SCORE_SCALED>, a, s256);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pose_score<256, VD_SCORE_UNIFORM>, a, s256);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pose_score<512, VD_SCORE_GENERAL>, a, s512);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pose_score<512, VD_SCORE_SCALED>, a, s512);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pose_score<512, VD_SCORE_UNIFORM>, a, s512);
   return e;
 }
 
@@ -1101,16 +1210,18 @@ cudaError_t launch_pose_score_only(vd_ctx* c) {
   const int nblk = std::max(1, c->score_bps * c->num_sms / 2);
   const dim3 grid(nblk, (M + 31) / 32);
   cudaError_t e = cudaSuccess;
-#define VD_SCORE_LAUNCH(TH, FAST)                                                              \
-  e = vd_launch(vd_overlap(c), k_pose_score<TH, FAST>, grid, TH, vd_score_smem(M, TH), c->stream, \
+#define VD_SCORE_LAUNCH(TH, MODE)                                                              \
+  e = vd_launch(vd_overlap(c), k_pose_score<TH, MODE>, grid, TH, vd_score_smem(M, TH), c->stream, \
                 P, c->rpts, c->robs, c->n_rigid, 0, c->rootsf, c->root_count, M, c->partial)
-  if (c->score_threads == 512) {
-    if (P.fast_beta2) VD_SCORE_LAUNCH(512, true);
-    else VD_SCORE_LAUNCH(512, false);
-  } else {
-    if (P.fast_beta2) VD_SCORE_LAUNCH(256, true);
-    else VD_SCORE_LAUNCH(256, false);
-  }
+#define VD_SCORE_MODES(TH)                                              \
+  do {                                                                  \
+    if (P.fast_beta2) VD_SCORE_LAUNCH(TH, VD_SCORE_UNIFORM);            \
+    else if (P.beta == 2.0f) VD_SCORE_LAUNCH(TH, VD_SCORE_SCALED);      \
+    else VD_SCORE_LAUNCH(TH, VD_SCORE_GENERAL);                         \
+  } while (0)
+  if (c->score_threads == 512) VD_SCORE_MODES(512);
+  else VD_SCORE_MODES(256);
+#undef VD_SCORE_MODES
 #undef VD_SCORE_LAUNCH
   if (e != cudaSuccess) return e;
   return launch_root_energy(vd_overlap(c), c->partial, nblk, M, c->root_count, c->root_energy, c->stream,
@@ -1229,6 +1340,23 @@ static cudaError_t noalloc_scratch(float** out, int* nblk) {
   return cudaSuccess;
 }
 
+// The scoring of a caller's points, each with its own scale in obs.z, and the
+// float64 sums.
+static cudaError_t launch_score_points(const DevParams& P, const float* points, const float* obs,
+                                       int n, const float* rootsf, int m, int nblk, size_t smem,
+                                       float* partial, double* energies, cudaStream_t s) {
+  const dim3 grid(nblk, (m + 31) / 32);
+  const float4 *pt = (const float4*)points, *ob = (const float4*)obs;
+  const cudaError_t e =
+      P.beta == 2.0f ? vd_launch(false, k_pose_score<SCORE_THREADS, VD_SCORE_SCALED>, grid,
+                                 SCORE_THREADS, smem, s, P, pt, ob, nullptr, n, rootsf, nullptr, m,
+                                 partial)
+                     : vd_launch(false, k_pose_score<SCORE_THREADS, VD_SCORE_GENERAL>, grid,
+                                 SCORE_THREADS, smem, s, P, pt, ob, nullptr, n, rootsf, nullptr, m,
+                                 partial);
+  return e != cudaSuccess ? e : launch_root_energy(true, partial, nblk, m, nullptr, energies, s);
+}
+
 extern "C" vd_status vd_score_poses_noalloc(const float* points, const float* obs, int n,
                                             const double* poses, int m, const double* intrinsics,
                                             float beta, float p0, double* energies,
@@ -1260,10 +1388,8 @@ extern "C" vd_status vd_score_poses_noalloc(const float* points, const float* ob
   float* rootsf = scratch;                                  // m x 12
   float* partial = scratch + 12 * VD_NOALLOC_MAX_POSES;     // m x nblk
   k_poses_float<<<(m + 127) / 128, 128, 0, s>>>(P, Kdev, poses, m, rootsf);
-  const size_t smem = vd_score_smem(m, SCORE_THREADS);
-  k_pose_score<SCORE_THREADS><<<dim3(nblk, (m + 31) / 32), SCORE_THREADS, smem, s>>>(
-      P, (const float4*)points, (const float4*)obs, nullptr, n, rootsf, nullptr, m, partial);
-  e = launch_root_energy(true, partial, nblk, m, nullptr, energies, s);
+  const size_t smem = vd_score_smem(m, SCORE_THREADS);   // 8 KB at most (m <= 1024)
+  e = launch_score_points(P, points, obs, n, rootsf, m, nblk, smem, partial, energies, s);
   cudaError_t e2 = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) {
@@ -1308,13 +1434,8 @@ extern "C" vd_status vd_score_poses(const float* points, const float* obs, int n
     return VD_ERR_OOM;
   }
   k_poses_float<<<(m + 127) / 128, 128, 0, s>>>(P, Kdev, poses, m, rootsf);
-  const size_t smem = vd_score_smem(m, SCORE_THREADS);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_pose_score<SCORE_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-  k_pose_score<SCORE_THREADS><<<dim3(nblk, (m + 31) / 32), SCORE_THREADS, smem, s>>>(
-      P, (const float4*)points, (const float4*)obs, nullptr, n, rootsf, nullptr, m, partial);
-  e = launch_root_energy(true, partial, nblk, m, nullptr, energies, s);
+  const size_t smem = vd_score_smem(m, SCORE_THREADS);   // 8 KB at most (m <= 1024)
+  e = launch_score_points(P, points, obs, n, rootsf, m, nblk, smem, partial, energies, s);
   cudaFreeAsync(rootsf, s);
   cudaError_t e2 = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = e2;
