@@ -169,6 +169,12 @@ __device__ __forceinline__ float vd_slot_candidate(const DevParams& P, uint32_t 
 // lowest slot.  Dropping a candidate whose partial key exceeds a pixel's best
 // key is exact: terms are non-negative, so its full key is at least the
 // partial key, and the best key is that of a finished candidate.
+// Bound: issue slots (71 % busy, the FMA pipe 24 %).  A term's x and y go
+// through packed float32 instructions (vd_f2, one slot for both), FAST leaves
+// the density's other form out of the code, and no term has a branch but the
+// one around its gather: the depth step of a 1216 x 368 window (N = 6, K =
+// 128, with the propagation) 715 -> 617 us, one of 509 x 383 pixels (N = 5, K =
+// 64, stereo prior) 278 -> 238 us, the results the same bits.
 // Ring bounds: the pre-pass runs only with fewer than 32 entries in ring 1
 // and adds at most 128; a stage-1 chunk runs only with fewer than 32 entries
 // in ring 2 and adds at most 32.
@@ -201,29 +207,31 @@ __device__ __forceinline__ unsigned vd_ring(int i) {
 
 // Flows [TA, TB) of one entry; false as soon as its partial energy exceeds
 // `thr`, the entry's drop threshold (see vd_drop_threshold).
-template <int TA, int TB>
+template <int TA, int TB, int NF, bool FAST>
 __device__ __forceinline__ bool vd_stage_terms(const DevParams& P, const float4 (*sTw)[32],
                                                const float4* sTail,
                                                const float2* __restrict__ flow, size_t npix,
                                                int p, float thr, float c, float& E, float& xp,
                                                float& yp) {
   const float NaN = __int_as_float(0x7fc00000);
+  const vd_f2 cc = vd_pack(c, c);
   VD_UNROLL(VD_KQ_STAGE_UNROLL)
   for (int t = TA; t < TB; ++t) {
     const float4 A = sTw[t - 1][p];
     const float4 M = sTail[t];
-    const float hx = fmaf(c, M.x, A.x);
-    const float hy = fmaf(c, M.y, A.y);
+    const vd_f2 h = vd_fma2(cc, vd_pack(M.x, M.y), vd_pack(A.x, A.y));
     const float hz = fmaf(c, M.z, A.z);
     const bool obs = vd_inside(xp, yp, P.W, P.H);   // false for NaN: behind camera t-1
-    float2 F = make_float2(0.0f, 0.0f);
-    if (obs) F = vd_bilinear(flow + (size_t)t * npix, P.W, P.H, xp, yp);
-    float x, y;
+    const vd_f2 xyp = vd_pack(xp, yp);
+    vd_f2 F = 0, xy;
+    if (obs) F = vd_bilinear2(flow + (size_t)t * npix, P.W, P.H, xyp);
     bool front;
-    const float l2 = vd_flow_term(P, hx, hy, hz, obs, F.x, F.y, xp, yp, &x, &y, &front);
+    const float l2 = t == NF - 1
+                         ? vd_flow_term2<FAST, VD_TERM_LAST>(P, h, hz, obs, F, xyp, &xy, &front)
+                         : vd_flow_term2<FAST, VD_TERM_INNER>(P, h, hz, obs, F, xyp, &xy, &front);
     E = fmaf(A.w, l2, E);
-    xp = front ? x : NaN;
-    yp = y;
+    xp = front ? vd_lo(xy) : NaN;
+    yp = vd_hi(xy);
     if (E > thr) return false;
   }
   return true;
@@ -240,7 +248,7 @@ __device__ __forceinline__ float vd_drop_threshold(unsigned long long best, unsi
   return bE <= 0.0f ? -1.0f : __int_as_float(__float_as_int(bE) - 1);
 }
 
-template <int NF, int WARPS>
+template <int NF, int WARPS, bool FAST>
 __global__ void __launch_bounds__(32 * WARPS, (4 * VD_KQ_MINB) / WARPS)
 k_depth_sample_q(DevParams P, const float* __restrict__ posef, const float2* __restrict__ flow,
                  const float* __restrict__ rho, const float* __restrict__ q,
@@ -315,7 +323,7 @@ k_depth_sample_q(DevParams P, const float* __restrict__ posef, const float2* __r
       const unsigned slot = id >> 5;
       const float thr = vd_drop_threshold(*(volatile unsigned long long*)&sBw[p], slot);
       float E = e.y, xp = e.z, yp = e.w;
-      if (vd_stage_terms<T1, NF>(P, sTw, sTail, flow, npix, p, thr, e.x, E, xp, yp))
+      if (vd_stage_terms<T1, NF, NF, FAST>(P, sTw, sTail, flow, npix, p, thr, e.x, E, xp, yp))
         atomicMin(&sBw[p], ((unsigned long long)__float_as_uint(E) << 32) | slot);
     }
     h2 = min(h2 + 32, e2);
@@ -336,19 +344,20 @@ VD_UNROLL(VD_KQ_PRE_UNROLL)
         cc = vd_clamp(cc, rmin, rmax);
         if (k == 1 && has_prior) cc = prior_c;
         float Ek = vd_prior_energy<NF>(px, P, cc);
-        const float hx = fmaf(cc, tail0.x, px.ax[0]);
-        const float hy = fmaf(cc, tail0.y, px.ay[0]);
+        const vd_f2 h = vd_fma2(vd_pack(cc, cc), vd_pack(tail0.x, tail0.y),
+                                vd_pack(px.ax[0], px.ay[0]));
         const float hz = fmaf(cc, tail0.z, px.az[0]);
-        float x1, y1;
+        vd_f2 xy1;
         bool f1;
-        const float l2 = vd_flow_term(P, hx, hy, hz, true, px.f1x, px.f1y, px.u, px.v, &x1, &y1, &f1);
+        const float l2 = vd_flow_term2<FAST, VD_TERM_INNER>(
+            P, h, hz, true, vd_pack(px.f1x, px.f1y), vd_pack(px.u, px.v), &xy1, &f1);
         Ek = fmaf(px.wl[0], l2, Ek);
         const unsigned long long key = ((unsigned long long)__float_as_uint(Ek) << 32) | (unsigned)k;
         const bool keep = valid && key < bnd;
         const unsigned m = __ballot_sync(FULL, keep);
         if (keep) {
           const unsigned pos = vd_ring<VD_KQ_R1>(e1 + __popc(m & lt));
-          sR1[wq][pos] = make_float4(cc, Ek, f1 ? x1 : NaN, y1);
+          sR1[wq][pos] = make_float4(cc, Ek, f1 ? vd_lo(xy1) : NaN, vd_hi(xy1));
           sI1[wq][pos] = (unsigned short)(lane | (k << 5));
         }
         e1 += __popc(m);
@@ -369,7 +378,8 @@ VD_UNROLL(VD_KQ_PRE_UNROLL)
         const int p = id & 31u;
         const unsigned slot = id >> 5;
         const float thr = vd_drop_threshold(*(volatile unsigned long long*)&sBw[p], slot);
-        keep = vd_stage_terms<1, T1>(P, sTw, sTail, flow, npix, p, thr, st.x, st.y, st.z, st.w);
+        keep = vd_stage_terms<1, T1, NF, FAST>(P, sTw, sTail, flow, npix, p, thr, st.x, st.y, st.z,
+                                             st.w);
         if (T1 == NF && keep)
           atomicMin(&sBw[p], ((unsigned long long)__float_as_uint(st.y) << 32) | slot);
       }
@@ -617,9 +627,17 @@ static cudaError_t launch_depth_sample_q(vd_ctx* c, uint32_t itcode, float s_per
   const dim3 blk(32 * WARPS);
   const dim3 grd((c->W + 31) / 32, (c->H + WARPS - 1) / WARPS);
   cudaError_t e = cudaSuccess;
-  VD_DISPATCH_NF2(nf, (e = vd_launch(vd_overlap(c), k_depth_sample_q<NF, WARPS>, grd, blk, 0, c->stream,
-                          c->dp, c->posef, c->flow, c->rho, c->q, c->prior_val, c->prior_rho,
-                          c->qhat, c->prior_conf, itcode, s_pert, c->rho_star, c->e_star)));
+#define VD_KQ_LAUNCH(FAST)                                                                       \
+  VD_DISPATCH_NF2(nf, (e = vd_launch(vd_overlap(c), k_depth_sample_q<NF, WARPS, FAST>, grd, blk, \
+                                     0, c->stream, c->dp, c->posef, c->flow, c->rho, c->q,       \
+                                     c->prior_val, c->prior_rho, c->qhat, c->prior_conf, itcode, \
+                                     s_pert, c->rho_star, c->e_star)))
+  if (c->dp.fast_beta2) {
+    VD_KQ_LAUNCH(true);
+  } else {
+    VD_KQ_LAUNCH(false);
+  }
+#undef VD_KQ_LAUNCH
   return e;
 }
 

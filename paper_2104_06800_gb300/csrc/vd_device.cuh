@@ -202,7 +202,7 @@ __device__ __forceinline__ float vd_ratio_y(const DevParams& P, float r2, float 
 // the residual-dependent part, so small y uses the series
 // ln(1 + y) = y - y^2/2 + y^3/3 - y^4/4 + y^5/5 (truncation < y^6/6).
 __device__ __forceinline__ float vd_ell2(float y) {
-  const float big = __log2f(1.0f + y);
+  const float big = vd_lg2(1.0f + y);
   const float ser =
       y * fmaf(y, fmaf(y, fmaf(y, fmaf(y, 0.2f, -0.25f), 0.33333334f), -0.5f), 1.0f) *
       1.44269504f;
@@ -230,10 +230,10 @@ __device__ __forceinline__ float vd_l2_general(const DevParams& P, float r2, flo
 __device__ __forceinline__ float vd_l2_beta2(const DevParams& P, float r2) {
   // beta = 2: P0 / p1 = P0 pi alpha^2 (1 + r^2 / alpha^2)^2
   const float s = fmaf(r2, P.inv_a2, 1.0f);
-  const float y = P.c0 * s * s;
+  const float y = __fmul_rn(__fmul_rn(P.c0, s), s);
   // one logarithm and no branch: of 1 + y, or of s where y would overflow
   const bool mid = y < 1e30f;
-  const float L = __log2f(mid ? 1.0f + y : s);
+  const float L = vd_lg2(mid ? __fadd_rn(1.0f, y) : s);
   const float ser =
       y * fmaf(y, fmaf(y, fmaf(y, fmaf(y, 0.2f, -0.25f), 0.33333334f), -0.5f), 1.0f) *
       1.44269504f;
@@ -263,18 +263,37 @@ __device__ __forceinline__ void vd_store_pose_entry(float* __restrict__ pf, floa
 // Bilinear sample of one flow field at (x, y), which must be inside the image.
 // Taps (x0, y0)..(x0+1, y0+1) with x0 = min(floor(x), W-2).
 // ---------------------------------------------------------------------------
+//
+// Both components go through packed arithmetic (vd_f2).  The floors come from
+// one packed addition of 2^23 rounded towards zero, which leaves floor(x) in
+// the low bits of each half for 0 <= x < 2^23 (images are at most 16384 wide
+// and high), in place of two conversions to integer and two back.
+__device__ __forceinline__ vd_f2 vd_bilinear2(const float2* __restrict__ F, int W, int H,
+                                              vd_f2 xy) {
+  const unsigned B = 0x4b000000u;                  // the bits of 2^23
+  const float two23 = 8388608.0f;
+  vd_f2 fl;
+  asm("add.rz.f32x2 %0, %1, %2;" : "=l"(fl) : "l"(xy), "l"(vd_pack(two23, two23)));
+  const unsigned x0 = min((unsigned)fl, B + (unsigned)(W - 2));
+  const unsigned y0 = min((unsigned)(fl >> 32), B + (unsigned)(H - 2));
+  const vd_f2 a = vd_sub2(xy, vd_sub2(vd_pack(__uint_as_float(x0), __uint_as_float(y0)),
+                                      vd_pack(two23, two23)));
+  // y0 W + x0 without the two 2^23 patterns, modulo 2^32
+  const unsigned i = y0 * (unsigned)W + (x0 - B * ((unsigned)W + 1u));
+  const float2* p = F + VD_CHK(VD_SITE_BILINEAR, (long long)i, (long long)W * H - W - 1);
+  const vd_f2* p0 = reinterpret_cast<const vd_f2*>(p);
+  const vd_f2* p1 = reinterpret_cast<const vd_f2*>(p + W);
+  const vd_f2 f00 = __ldg(p0), f01 = __ldg(p0 + 1);
+  const vd_f2 f10 = __ldg(p1), f11 = __ldg(p1 + 1);
+  const vd_f2 ax = vd_pack(vd_lo(a), vd_lo(a)), ay = vd_pack(vd_hi(a), vd_hi(a));
+  const vd_f2 t = vd_fma2(ax, vd_sub2(f01, f00), f00);
+  const vd_f2 b = vd_fma2(ax, vd_sub2(f11, f10), f10);
+  return vd_fma2(ay, vd_sub2(b, t), t);
+}
 __device__ __forceinline__ float2 vd_bilinear(const float2* __restrict__ F, int W, int H, float x,
                                               float y) {
-  const int x0 = min(__float2int_rd(x), W - 2);
-  const int y0 = min(__float2int_rd(y), H - 2);
-  const float ax = x - (float)x0;
-  const float ay = y - (float)y0;
-  const float2* p = F + VD_CHK(VD_SITE_BILINEAR, (long long)y0 * W + x0, (long long)W * H - W - 1);
-  const float2 f00 = __ldg(p), f01 = __ldg(p + 1);
-  const float2 f10 = __ldg(p + W), f11 = __ldg(p + W + 1);
-  const float tx = fmaf(ax, f01.x - f00.x, f00.x), ty = fmaf(ax, f01.y - f00.y, f00.y);
-  const float bx = fmaf(ax, f11.x - f10.x, f10.x), by = fmaf(ax, f11.y - f10.y, f10.y);
-  return make_float2(fmaf(ay, bx - tx, tx), fmaf(ay, by - ty, ty));
+  const vd_f2 r = vd_bilinear2(F, W, H, vd_pack(x, y));
+  return make_float2(vd_lo(r), vd_hi(r));
 }
 
 __device__ __forceinline__ bool vd_inside(float x, float y, int W, int H) {
@@ -346,30 +365,41 @@ __device__ __forceinline__ float vd_prior_energy(const VdPixel<NF>& px, const De
   return px.pw * (z > 20.0f ? z : VD_LN2 * vd_ell2(__expf(z)));
 }
 
-// One flow term in log2 units.  (hx, hy, hz): homogeneous image point of the
-// candidate in frame t; (xp, yp): its image point in frame t-1, where the
-// flow (Fx, Fy) was read; obs: the point is in front of camera t-1 and
+// One flow term in log2 units.  (h, hz): homogeneous image point of the
+// candidate in frame t, x and y packed; xyp: its image point in frame t-1,
+// where the flow F was read; obs: the point is in front of camera t-1 and
 // inside image t-1.  Writes the image point in frame t and whether it is in
-// front of camera t.
-__device__ __forceinline__ float vd_flow_term(const DevParams& P, float hx, float hy, float hz,
-                                              bool obs, float Fx, float Fy, float xp, float yp,
-                                              float* x_out, float* y_out, bool* front_out) {
+// front of camera t.  Without a branch: a term is almost always observed, and
+// what is not is discarded.  FAST: the launch's constants (beta = 2, one
+// scale for all pixels).  POS: the window's last flow has an image point that
+// nothing else reads; its products are scalar, since the compiler fuses a
+// packed product into the packed difference that alone uses it.  The only flow
+// of a window (and of the bootstrap's own depth) has that displacement in one
+// multiply-add.
+enum { VD_TERM_INNER = 0, VD_TERM_LAST = 1, VD_TERM_ONLY = 2 };
+template <bool FAST, int POS>
+__device__ __forceinline__ float vd_flow_term2(const DevParams& P, vd_f2 h, float hz, bool obs,
+                                               vd_f2 F, vd_f2 xyp, vd_f2* xy_out,
+                                               bool* front_out) {
   const bool front = hz > VD_Z_EPS;
-  const float iz = __fdividef(1.0f, hz);
-  const float x = hx * iz, y = hy * iz;
-  float l2;
-  if (obs && front) {
-    const float dx = Fx - (x - xp);
-    const float dy = Fy - (y - yp);
-    const float r2 = fmaf(dx, dx, dy * dy);
-    l2 = vd_l2_flow(P, r2, fmaf(Fx, Fx, Fy * Fy));
-  } else {
-    l2 = obs ? (VD_L_BEHIND / VD_LN2) : 0.0f;
-  }
-  *x_out = x;
-  *y_out = y;
+  const float r = vd_rcp(hz);
+  *xy_out = POS == VD_TERM_LAST ? vd_pack(__fmul_rn(vd_lo(h), r), __fmul_rn(vd_hi(h), r))
+                                : vd_mul2(h, vd_pack(r, r));
   *front_out = front;
-  return l2;
+  const vd_f2 d =
+      vd_sub2(F, POS == VD_TERM_ONLY
+                     ? vd_fma2(h, vd_pack(r, r), vd_pack(-vd_lo(xyp), -vd_hi(xyp)))
+                     : vd_sub2(*xy_out, xyp));
+  const float dx = vd_lo(d), dy = vd_hi(d);
+  const float r2 = fmaf(dx, dx, dy * dy);
+  float l2;
+  if (FAST) {
+    l2 = vd_l2_beta2(P, r2);
+  } else {
+    const float Fx = vd_lo(F), Fy = vd_hi(F);
+    l2 = vd_l2_general(P, r2, fmaf(P.alpha1, sqrtf(fmaf(Fx, Fx, Fy * Fy)), P.alpha0));
+  }
+  return obs ? (front ? l2 : VD_L_BEHIND / VD_LN2) : 0.0f;
 }
 
 // E_j(c) in full, for latency-bound callers (the chain propagation): every
@@ -451,34 +481,33 @@ __device__ __forceinline__ float vd_energy(const VdPixel<NF>& px, const DevParam
                                            const float2* __restrict__ flow, size_t npix,
                                            float c, float bound = INFINITY) {
   float E = vd_prior_energy<NF>(px, P, c);
-  float xp = px.u, yp = px.v;
+  vd_f2 xyp = vd_pack(px.u, px.v);
   bool front_prev = true;
 #pragma unroll
   for (int t = 0; t < NF; ++t) {
     if (E >= bound) return E;
     const float* M = sPose + 12 * (t + 1);
-    const float hx = fmaf(c, M[9], px.ax[t]);
-    const float hy = fmaf(c, M[10], px.ay[t]);
+    const vd_f2 h = vd_pack(fmaf(c, M[9], px.ax[t]), fmaf(c, M[10], px.ay[t]));
     const float hz = fmaf(c, M[11], px.az[t]);
-    bool obs;
-    float Fx, Fy;
-    if (t == 0) {
-      obs = true;
-      Fx = px.f1x;
-      Fy = px.f1y;
-    } else {
-      obs = front_prev && vd_inside(xp, yp, P.W, P.H);
-      float2 F = make_float2(0.0f, 0.0f);
-      if (obs) F = vd_bilinear(flow + (size_t)t * npix, P.W, P.H, xp, yp);
-      Fx = F.x;
-      Fy = F.y;
+    bool obs = true;
+    vd_f2 F = vd_pack(px.f1x, px.f1y);
+    if (t > 0) {
+      obs = front_prev && vd_inside(vd_lo(xyp), vd_hi(xyp), P.W, P.H);
+      F = 0;
+      if (obs) F = vd_bilinear2(flow + (size_t)t * npix, P.W, P.H, xyp);
     }
-    float x, y;
+    vd_f2 xy;
     bool front;
-    const float l2 = vd_flow_term(P, hx, hy, hz, obs, Fx, Fy, xp, yp, &x, &y, &front);
+    float l2;
+    constexpr int END = NF == 1 ? VD_TERM_ONLY : VD_TERM_LAST;
+    if (t == NF - 1)
+      l2 = P.fast_beta2 ? vd_flow_term2<true, END>(P, h, hz, obs, F, xyp, &xy, &front)
+                        : vd_flow_term2<false, END>(P, h, hz, obs, F, xyp, &xy, &front);
+    else
+      l2 = P.fast_beta2 ? vd_flow_term2<true, VD_TERM_INNER>(P, h, hz, obs, F, xyp, &xy, &front)
+                        : vd_flow_term2<false, VD_TERM_INNER>(P, h, hz, obs, F, xyp, &xy, &front);
     E = fmaf(px.wl[t], l2, E);
-    xp = x;
-    yp = y;
+    xyp = xy;
     front_prev = front;
   }
   return E;
