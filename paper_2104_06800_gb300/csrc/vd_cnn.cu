@@ -1001,6 +1001,11 @@ struct vd_cnn {
   int* nmask;          // pixels inside the training mask
   double* geo;         // [12] T_1 given to the host-API calls
   int* err;
+  // CTAs of the persistent kernels that are resident at once on the network's
+  // device (cnn_prepare)
+  int slots_in, slots_hid, slots_last;   // forward: layer 1 of 16 planes, 32 planes, last
+  int slots_dlast, slots_dhid;           // data gradient of the last layer, of the others
+  int slots_wg;
 };
 
 static void cnn_free_images(vd_cnn* n) {
@@ -1064,27 +1069,55 @@ static cudaError_t vd_image_map(CUtensorMap* m, const void* X, int ch, int W, in
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// Grants a convolution its shared memory on the current device and counts the
+// CTAs that fit on it at once, the persistent grid.
+template <int K, int N, int EPI>
+static cudaError_t conv_prepare(int sms, int* slots) {
+  using S = VdConvShape<K, N, CNN_ROWS, CNN_STAGES>;
+  auto kern = k_conv_tc<K, N, EPI, CNN_ROWS, CNN_STAGES>;
+  int per_sm = 0;
+  cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, CNN_CONV_THREADS, S::SMEM);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  *slots = sms * per_sm;
+  return cudaSuccess;
+}
+
+template <int CIN, int COUT>
+static cudaError_t wgrad_prepare() {
+  return cudaFuncSetAttribute(k_wgrad_tc<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)VdWgradShape<CIN, COUT>::SMEM);
+}
+
+// Function attributes and grid sizes of the network's kernels on the device it
+// is created on.  Kept with the network, not with the process: attributes and
+// SM counts are a device's, and end with its context.
+static cudaError_t cnn_prepare(vd_cnn* n) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = conv_prepare<144, 32, EPI_RELU>(sms, &n->slots_in);
+  if (e == cudaSuccess) e = conv_prepare<288, 32, EPI_RELU>(sms, &n->slots_hid);
+  if (e == cudaSuccess) e = conv_prepare<288, 16, EPI_LAST>(sms, &n->slots_last);
+  if (e == cudaSuccess) e = conv_prepare<144, 32, EPI_DGRAD>(sms, &n->slots_dlast);
+  if (e == cudaSuccess) e = conv_prepare<288, 32, EPI_DGRAD>(sms, &n->slots_dhid);
+  if (e == cudaSuccess) e = wgrad_prepare<32, 16>();
+  if (e == cudaSuccess) e = wgrad_prepare<16, 32>();
+  if (e == cudaSuccess) e = wgrad_prepare<32, 32>();
+  n->slots_wg = min(sms, WG_MAX_BLOCKS);   // one CTA per SM
+  return e;
+}
+
 template <int K, int N, int EPI>
 static cudaError_t launch_conv(const __nv_bfloat16* X, int W, int H, const __nv_bfloat16* Wt,
                                const float* b, void* out, const __nv_bfloat16* mask, int* err,
-                               cudaStream_t s, int nout = N) {
+                               int slots, cudaStream_t s, int nout = N) {
   constexpr int R = CNN_ROWS, NS = CNN_STAGES;
   using S = VdConvShape<K, N, R, NS>;
   auto kern = k_conv_tc<K, N, EPI, R, NS>;
-  // persistent grid: every CTA that fits on the device at once (set up once)
-  static int slots = 0;
-  if (!slots) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, CNN_CONV_THREADS, S::SMEM);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    slots = sms * per_sm;
-  }
   CUtensorMap map;
   cudaError_t e = vd_image_map(&map, X, K / 9, W, H, CNN_HALO_X, R + 2);
   if (e != cudaSuccess) return e;
@@ -1117,13 +1150,13 @@ static cudaError_t cnn_forward(vd_cnn* n, const float* flow, int W, int H, cudaS
     const int K = 9 * n->cin[l];
     if (l == CNN_L - 1) {
       e = launch_conv<288, 16, EPI_LAST>(n->act[l], W, H, n->wt[l], b, n->zlast, nullptr, n->err,
-                                         s, n->cout[l]);
+                                         n->slots_last, s, n->cout[l]);
     } else if (K == 144) {
       e = launch_conv<144, 32, EPI_RELU>(n->act[l], W, H, n->wt[l], b, n->act[l + 1], nullptr,
-                                         n->err, s);
+                                         n->err, n->slots_in, s);
     } else {
       e = launch_conv<288, 32, EPI_RELU>(n->act[l], W, H, n->wt[l], b, n->act[l + 1], nullptr,
-                                         n->err, s);
+                                         n->err, n->slots_hid, s);
     }
     if (e != cudaSuccess) return e;
   }
@@ -1138,22 +1171,12 @@ static cudaError_t launch_wgrad(vd_cnn* n, int l, const __nv_bfloat16* dz, int W
                                 cudaStream_t s) {
   using S = VdWgradShape<CIN, COUT>;
   auto kern = k_wgrad_tc<CIN, COUT>;
-  static int slots = 0;   // persistent grid: one CTA per SM (set up once)
-  if (!slots) {
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
-    if (e != cudaSuccess) return e;
-    slots = min(sms, WG_MAX_BLOCKS);
-  }
   CUtensorMap xmap, dmap;
   cudaError_t e = vd_image_map(&xmap, n->act[l], CIN, W, H, CNN_HALO_X, WG_ROWS);
   if (e == cudaSuccess) e = vd_image_map(&dmap, dz, COUT, W, H, CNN_TILE, WG_ROWS + 2);
   if (e != cudaSuccess) return e;
   const int tiles_x = (W + CNN_TILE - 1) / CNN_TILE;
-  const int n_tiles = tiles_x * ((H + WG_ROWS - 1) / WG_ROWS), nblk = min(n_tiles, slots);
+  const int n_tiles = tiles_x * ((H + WG_ROWS - 1) / WG_ROWS), nblk = min(n_tiles, n->slots_wg);
   e = vd_launch(true, kern, nblk, WG_THREADS, S::SMEM, s, xmap, dmap, W, H, tiles_x, n_tiles,
                 n->wg_partial, n->wg_partial_b, n->err);
   if (e != cudaSuccess) return e;
@@ -1177,9 +1200,11 @@ static cudaError_t cnn_backward(vd_cnn* n, int W, int H, cudaStream_t s) {
     if (e != cudaSuccess || l == 0) break;
     // dL/dz_{l-1} = (W_l^T * dL/dz_l) where a_l > 0
     if (l == CNN_L - 1)
-      e = launch_conv<144, 32, EPI_DGRAD>(dz, W, H, n->wd[l], nullptr, nxt, n->act[l], n->err, s);
+      e = launch_conv<144, 32, EPI_DGRAD>(dz, W, H, n->wd[l], nullptr, nxt, n->act[l], n->err,
+                                          n->slots_dlast, s);
     else
-      e = launch_conv<288, 32, EPI_DGRAD>(dz, W, H, n->wd[l], nullptr, nxt, n->act[l], n->err, s);
+      e = launch_conv<288, 32, EPI_DGRAD>(dz, W, H, n->wd[l], nullptr, nxt, n->act[l], n->err,
+                                          n->slots_dhid, s);
     __nv_bfloat16* t = dz;
     dz = nxt;
     nxt = t;
@@ -1277,7 +1302,8 @@ extern "C" vd_status vd_cnn_create(int n_flows, unsigned long long seed, vd_cnn*
               ci < cin_real ? (float)(g * sd) : 0.0f;
         }
   }
-  cudaError_t e = cudaMalloc(&n->theta, sizeof(float) * off);
+  cudaError_t e = cnn_prepare(n);
+  if (e == cudaSuccess) e = cudaMalloc(&n->theta, sizeof(float) * off);
   if (e == cudaSuccess) e = cudaMalloc(&n->mom1, sizeof(float) * off);
   if (e == cudaSuccess) e = cudaMalloc(&n->mom2, sizeof(float) * off);
   if (e == cudaSuccess) e = cudaMalloc(&n->grad, sizeof(float) * off);
