@@ -184,6 +184,9 @@ vd_status vd_get_pose_samples(vd_ctx* ctx, double* poses, double* energies, int*
  * with points[i] = (X, Y, Z, w) and obs[i] = (x, y, alpha, unused) as float4,
  * l the Fisk maximum-inlier energy with shape beta and outlier density p0,
  * and a large constant for points behind the camera.  energies: m float64.
+ * points, obs, poses and energies are device memory, read and written in the
+ * order of cuda_stream.  intrinsics: 4 float64 (fx, fy, cx, cy) in host or
+ * device memory, read after all earlier work of the default stream too.
  * Allocates its own scratch for the block partial sums; runs on cuda_stream
  * and synchronises it.  n >= 0 (points and obs may be NULL when n = 0, which
  * gives zero energies), 1 <= m <= 1024. */

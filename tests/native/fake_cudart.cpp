@@ -32,6 +32,7 @@ std::map<void*, Block> g_blocks;
 std::map<void*, Pool> g_pools;
 std::map<std::pair<int, const void*>, int> g_smem;
 std::map<const void*, std::string> g_names;
+std::map<const void*, std::pair<size_t, void*>> g_symbols;   // size, device address
 int g_launches, g_dead_pool_uses, g_blocking_copies;
 unsigned g_max_persistent_grid;
 const double* g_last_K;          // k_poses_float's second argument
@@ -134,7 +135,15 @@ void __cudaRegisterFunction(void**, const char* host, char*, const char* name, i
                             dim3*, dim3*, int*) {
   g_names[host] = name;
 }
-void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
+void __cudaRegisterVar(void**, char* host, char*, const char*, int, size_t n, int, int) {
+  g_symbols[host] = {n, nullptr};
+}
+cudaError_t cudaGetSymbolAddress(void** p, const void* host) {
+  auto& v = g_symbols[host];
+  if (!v.second) v.second = aligned_alloc(256, (v.first + 255) / 256 * 256);
+  *p = v.second;
+  return cudaSuccess;
+}
 
 // launches
 static dim3 s_grid, s_block;
