@@ -188,7 +188,10 @@ vd_status vd_get_pose_samples(vd_ctx* ctx, double* poses, double* energies, int*
  * order of cuda_stream.  intrinsics: 4 float64 (fx, fy, cx, cy) in host or
  * device memory, read after all earlier work of the default stream too.
  * Allocates its own scratch for the block partial sums; runs on cuda_stream
- * and synchronises it.  n >= 0 (points and obs may be NULL when n = 0, which
+ * and synchronises it.  The scratch of this call and of vd_ka_align comes from
+ * a memory pool of the library's, which keeps up to 32 MB per device for the
+ * next call until the process exits; a device allocation of the library that
+ * finds no memory gives it back first.  n >= 0 (points and obs may be NULL when n = 0, which
  * gives zero energies), 1 <= m <= 1024. */
 vd_status vd_score_poses(const float* points, const float* obs, int n, const double* poses, int m,
                          const double* intrinsics, float beta, float p0, double* energies,
@@ -456,7 +459,8 @@ vd_status vd_get_frame_samples(vd_ctx* ctx, int t, double* poses, double* energi
  * lowers E (lambda /= 10), refused otherwise (lambda *= 10); lambda starts at
  * 1e-3; stop after max_iters steps, a step below 1e-10, or lambda > 1e10.
  * cov = the pose block of H^-1 (rotation first), NaN without a pixel.
- * Device buffers; float64 arithmetic.  Synchronises the stream. */
+ * Device buffers; float64 arithmetic.  Synchronises the stream.  Scratch as
+ * vd_score_poses. */
 typedef struct {
   double pose[12];   /* T; in: start, 3x4 keyframe-2 -> keyframe-1; out: estimate */
   double s;          /* in: start (> 0); out: estimate                          */

@@ -24,8 +24,10 @@ extern "C" const char* vd_last_error(void) { return g_err; }
 // stream-ordered pool of the library's own, one per device.  The device's
 // default pool gives its memory back at every synchronisation, and each of
 // these calls ends with one, so that every call mapped its scratch anew (0.18
-// ms of a 0.44 ms scoring call); this pool keeps up to VD_WS_KEEP bytes, and
-// an allocation that finds no memory gives all of it back and tries again.
+// ms of a 0.44 ms scoring call); this pool keeps up to VD_WS_KEEP bytes, the
+// scratch of an alignment of about 1000 x 1000 pixels (32 bytes each), above
+// which a call maps what is beyond it anew.  Every device allocation of the
+// library that finds no memory gives all of it back and tries again.
 // Allocation and release are ordered by their stream and safe from several
 // threads; the pool itself is created once per device under a lock.
 // ---------------------------------------------------------------------------
@@ -67,6 +69,7 @@ cudaError_t vd_ws_alloc(void** p, size_t bytes, cudaStream_t s) {
     cudaMemPoolTrimTo(pool, 0);
     e = cudaMallocFromPoolAsync(p, bytes, pool, s);
   }
+  if (e != cudaSuccess) cudaGetLastError();   // returned, and left nowhere else
   return e;
 }
 
@@ -76,6 +79,17 @@ static void ws_trim() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= VD_WS_DEVICES) return;
   std::lock_guard<std::mutex> lock(g_ws_mu);
   if (g_ws_pool[dev]) cudaMemPoolTrimTo(g_ws_pool[dev], 0);
+}
+
+cudaError_t vd_device_alloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    ws_trim();
+    e = cudaMalloc(p, bytes);
+  }
+  if (e != cudaSuccess) cudaGetLastError();   // returned, and left nowhere else
+  return e;
 }
 
 // ---------------------------------------------------------------------------
@@ -283,13 +297,7 @@ static void fill_devparams(vd_ctx* c) {
 
 template <typename T>
 static cudaError_t dalloc(T** p, size_t n) {
-  cudaError_t e = cudaMalloc((void**)p, sizeof(T) * (n ? n : 1));
-  if (e == cudaErrorMemoryAllocation) {
-    cudaGetLastError();
-    ws_trim();
-    e = cudaMalloc((void**)p, sizeof(T) * (n ? n : 1));
-  }
-  return e;
+  return vd_malloc(p, sizeof(T) * (n ? n : 1));
 }
 
 extern "C" vd_status vd_destroy(vd_ctx* c) {
@@ -1023,7 +1031,7 @@ extern "C" vd_status vd_batch_create(int n, const vd_window_desc* descs, const v
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     if (e == cudaSuccess) b->join.push_back(ev);
   }
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_deg, sizeof(int) * n);
+  if (e == cudaSuccess) e = vd_malloc(&b->d_deg, sizeof(int) * n);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_deg, sizeof(int) * n);
   if (e != cudaSuccess) {
     vd_set_error(cudaGetErrorString(e));

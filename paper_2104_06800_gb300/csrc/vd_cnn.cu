@@ -1025,11 +1025,11 @@ static cudaError_t cnn_reserve(vd_cnn* n, int HW) {
   cnn_free_images(n);
   cudaError_t e = cudaSuccess;
   for (int l = 0; l < CNN_L && e == cudaSuccess; ++l)
-    e = cudaMalloc(&n->act[l], sizeof(__nv_bfloat16) * (size_t)HW * n->cin[l]);
-  if (e == cudaSuccess) e = cudaMalloc(&n->g0, sizeof(__nv_bfloat16) * (size_t)HW * CNN_WIDTH);
-  if (e == cudaSuccess) e = cudaMalloc(&n->g1, sizeof(__nv_bfloat16) * (size_t)HW * CNN_WIDTH);
-  if (e == cudaSuccess) e = cudaMalloc(&n->zlast, sizeof(float) * 16 * (size_t)HW);
-  if (e == cudaSuccess) e = cudaMalloc(&n->loss_partial, sizeof(double) * ((HW + 255) / 256));
+    e = vd_malloc(&n->act[l], sizeof(__nv_bfloat16) * (size_t)HW * n->cin[l]);
+  if (e == cudaSuccess) e = vd_malloc(&n->g0, sizeof(__nv_bfloat16) * (size_t)HW * CNN_WIDTH);
+  if (e == cudaSuccess) e = vd_malloc(&n->g1, sizeof(__nv_bfloat16) * (size_t)HW * CNN_WIDTH);
+  if (e == cudaSuccess) e = vd_malloc(&n->zlast, sizeof(float) * 16 * (size_t)HW);
+  if (e == cudaSuccess) e = vd_malloc(&n->loss_partial, sizeof(double) * ((HW + 255) / 256));
   if (e == cudaSuccess) n->cap_hw = HW;
   return e;
 }
@@ -1303,23 +1303,23 @@ extern "C" vd_status vd_cnn_create(int n_flows, unsigned long long seed, vd_cnn*
         }
   }
   cudaError_t e = cnn_prepare(n);
-  if (e == cudaSuccess) e = cudaMalloc(&n->theta, sizeof(float) * off);
-  if (e == cudaSuccess) e = cudaMalloc(&n->mom1, sizeof(float) * off);
-  if (e == cudaSuccess) e = cudaMalloc(&n->mom2, sizeof(float) * off);
-  if (e == cudaSuccess) e = cudaMalloc(&n->grad, sizeof(float) * off);
+  if (e == cudaSuccess) e = vd_malloc(&n->theta, sizeof(float) * off);
+  if (e == cudaSuccess) e = vd_malloc(&n->mom1, sizeof(float) * off);
+  if (e == cudaSuccess) e = vd_malloc(&n->mom2, sizeof(float) * off);
+  if (e == cudaSuccess) e = vd_malloc(&n->grad, sizeof(float) * off);
   for (int l = 0; l < CNN_L && e == cudaSuccess; ++l) {
     const int npad = n->cout[l] < 16 ? 16 : n->cout[l];
-    e = cudaMalloc(&n->wt[l], sizeof(__nv_bfloat16) * npad * 9 * n->cin[l]);
+    e = vd_malloc(&n->wt[l], sizeof(__nv_bfloat16) * npad * 9 * n->cin[l]);
     if (e == cudaSuccess && l > 0)
-      e = cudaMalloc(&n->wd[l], sizeof(__nv_bfloat16) * n->cin[l] * 9 * npad);
+      e = vd_malloc(&n->wd[l], sizeof(__nv_bfloat16) * n->cin[l] * 9 * npad);
   }
   if (e == cudaSuccess)
-    e = cudaMalloc(&n->wg_partial, sizeof(float) * WG_MAX_BLOCKS * CNN_WIDTH * 9 * CNN_WIDTH);
-  if (e == cudaSuccess) e = cudaMalloc(&n->wg_partial_b, sizeof(float) * WG_MAX_BLOCKS * CNN_WIDTH);
-  if (e == cudaSuccess) e = cudaMalloc(&n->loss, sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&n->nmask, sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&n->err, sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&n->geo, sizeof(double) * 12);
+    e = vd_malloc(&n->wg_partial, sizeof(float) * WG_MAX_BLOCKS * CNN_WIDTH * 9 * CNN_WIDTH);
+  if (e == cudaSuccess) e = vd_malloc(&n->wg_partial_b, sizeof(float) * WG_MAX_BLOCKS * CNN_WIDTH);
+  if (e == cudaSuccess) e = vd_malloc(&n->loss, sizeof(double));
+  if (e == cudaSuccess) e = vd_malloc(&n->nmask, sizeof(int));
+  if (e == cudaSuccess) e = vd_malloc(&n->err, sizeof(int));
+  if (e == cudaSuccess) e = vd_malloc(&n->geo, sizeof(double) * 12);
   if (e == cudaSuccess) e = cudaMemcpy(n->theta, h.data(), sizeof(float) * off, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(n->mom1, 0, sizeof(float) * off);
   if (e == cudaSuccess) e = cudaMemset(n->mom2, 0, sizeof(float) * off);

@@ -181,6 +181,14 @@ void vd_set_error(const char* msg);
 // stream.
 cudaError_t vd_ws_alloc(void** p, size_t bytes, cudaStream_t s);
 
+// Device memory of a context, network or batch; without room, the scratch kept
+// for the standalone calls is given back first.
+cudaError_t vd_device_alloc(void** p, size_t bytes);
+template <typename T>
+static inline cudaError_t vd_malloc(T** p, size_t bytes) {
+  return vd_device_alloc((void**)p, bytes);
+}
+
 // Return from a vd_status function on a CUDA error (recording its message).
 #define VD_CU(call)                                   \
   do {                                                \
