@@ -1,12 +1,16 @@
 // Host runtime of the library: context lifecycle, input upload, the EM
 // schedule of VOLDOR+ (Sec. III-A) and result download.  Every function is
 // a C-ABI entry point declared in voldor_em.h.
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
 
 #include <algorithm>
+#include <map>
 #include <mutex>
+#include <utility>
 #include <vector>
 
 #include "vd_internal.h"
@@ -29,63 +33,74 @@ extern "C" const char* vd_last_error(void) { return g_err; }
 // which a call maps what is beyond it anew.  Every device allocation of the
 // library that finds no memory gives all of it back and tries again.
 // Allocation and release are ordered by their stream and safe from several
-// threads; the pool itself is created once per device under a lock.
+// threads; the pool itself is created once per device and context under a lock,
+// and where none can be made the default pool serves.
 // ---------------------------------------------------------------------------
 #define VD_WS_KEEP (32ull << 20)
-#define VD_WS_DEVICES 64
 static std::mutex g_ws_mu;
-static cudaMemPool_t g_ws_pool[VD_WS_DEVICES];
+// by device and context (a reset leaves its handle behind, which no context
+// finds any more)
+static std::map<std::pair<int, unsigned long long>, cudaMemPool_t> g_ws_pools;
+
+// Identity of the current context, unique in the process (the next one of a
+// device that was reset has another), or 0 where the driver does not tell.
+static unsigned long long context_id() {
+  static const PFN_cuCtxGetId_v12000 get = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+    const cudaError_t e =
+        cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q);
+    return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? (PFN_cuCtxGetId_v12000)f
+                                                                : nullptr;
+  }();
+  unsigned long long id = 0;
+  if (!get) return 0;
+  if (get(nullptr, &id) == CUDA_SUCCESS) return id;
+  cudaFree(nullptr);   // no context yet, or none since a reset: the runtime makes one
+  return get(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// The pool of the current device and context (made if `make`), or null.
+static cudaMemPool_t ws_pool(bool make) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  std::lock_guard<std::mutex> lock(g_ws_mu);
+  const std::pair<int, unsigned long long> key(dev, context_id());
+  const auto it = g_ws_pools.find(key);
+  if (it != g_ws_pools.end() || !make) return it != g_ws_pools.end() ? it->second : nullptr;
+  cudaMemPoolProps props;
+  memset(&props, 0, sizeof props);
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  cudaMemPool_t made = nullptr;
+  unsigned long long keep = VD_WS_KEEP;
+  if (cudaMemPoolCreate(&made, &props) != cudaSuccess) return nullptr;
+  if (cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    cudaMemPoolDestroy(made);
+    return nullptr;
+  }
+  return g_ws_pools[key] = made;
+}
 
 cudaError_t vd_ws_alloc(void** p, size_t bytes, cudaStream_t s) {
   *p = nullptr;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= VD_WS_DEVICES) return cudaMallocAsync(p, bytes, s);
-  cudaMemPool_t pool = nullptr;
-  {
-    std::lock_guard<std::mutex> lock(g_ws_mu);
-    if (!g_ws_pool[dev]) {
-      cudaMemPoolProps props;
-      memset(&props, 0, sizeof props);
-      props.allocType = cudaMemAllocationTypePinned;
-      props.location.type = cudaMemLocationTypeDevice;
-      props.location.id = dev;
-      cudaMemPool_t made = nullptr;
-      unsigned long long keep = VD_WS_KEEP;
-      if ((e = cudaMemPoolCreate(&made, &props)) != cudaSuccess) return e;
-      if ((e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep)) !=
-          cudaSuccess) {
-        cudaMemPoolDestroy(made);
-        return e;
-      }
-      g_ws_pool[dev] = made;
-    }
-    pool = g_ws_pool[dev];
-  }
-  e = cudaMallocFromPoolAsync(p, bytes, pool, s);
-  if (e == cudaErrorMemoryAllocation) {
+  const cudaMemPool_t pool = ws_pool(true);
+  cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+  if (pool && e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
     cudaMemPoolTrimTo(pool, 0);
     e = cudaMallocFromPoolAsync(p, bytes, pool, s);
   }
-  if (e != cudaSuccess) cudaGetLastError();   // returned, and left nowhere else
+  if (e != cudaSuccess || !pool) cudaGetLastError();   // returned, and left nowhere else
   return e;
-}
-
-// Gives back what the current device's pool keeps unused.
-static void ws_trim() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= VD_WS_DEVICES) return;
-  std::lock_guard<std::mutex> lock(g_ws_mu);
-  if (g_ws_pool[dev]) cudaMemPoolTrimTo(g_ws_pool[dev], 0);
 }
 
 cudaError_t vd_device_alloc(void** p, size_t bytes) {
   cudaError_t e = cudaMalloc(p, bytes);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
-    ws_trim();
+    if (const cudaMemPool_t pool = ws_pool(false)) cudaMemPoolTrimTo(pool, 0);
     e = cudaMalloc(p, bytes);
   }
   if (e != cudaSuccess) cudaGetLastError();   // returned, and left nowhere else

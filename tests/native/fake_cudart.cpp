@@ -115,6 +115,7 @@ void fake_capacity(size_t bytes) { g_capacity = bytes; }
 size_t fake_used(int dev) { return g_used[dev]; }
 size_t fake_idle(int dev) { return idle_bytes(dev); }
 int fake_dead_pool_uses() { return g_dead_pool_uses; }
+int fake_pools() { return (int)g_pools.size(); }
 int fake_blocking_copies() { return g_blocking_copies; }
 unsigned fake_max_persistent_grid() { return g_max_persistent_grid; }
 int fake_intrinsics(double* K) {   // what k_poses_float read; 1: by pointer, 0: none, -1: misaligned

@@ -86,3 +86,32 @@ fake.fake_capacity(fake.fake_used(0) + 1000)
 assert lib.vd_score_poses(pts, obs, n, poses, m, K, F(2.0), F(1e-3), out, None) == -3
 assert fake.cudaGetLastError() == 0
 """)
+
+
+def test_calls_after_a_device_reset():
+    """A reset ends the pool with its context; neither call may use it again."""
+    fake_cuda.run(ALIGN + """
+for call in (score, align):
+    call()
+    assert fake.cudaDeviceReset() == 0
+    call()
+    assert fake.fake_dead_pool_uses() == 0
+# the allocations that would trim the dead pool
+assert fake.cudaDeviceReset() == 0
+fake.fake_capacity(1000)
+net = P()
+assert lib.vd_cnn_create(6, C.c_ulonglong(0), C.byref(net)) == -3
+assert fake.fake_dead_pool_uses() == 0
+""")
+
+
+def test_one_pool_per_device():
+    fake_cuda.run(ALIGN + """
+for d in (0, 1, 0, 1, 0):
+    assert fake.cudaSetDevice(d) == 0
+    align()
+    score()
+assert fake.fake_pools() == 2 and fake.fake_dead_pool_uses() == 0
+for d in (0, 1):
+    assert 0 < fake.fake_idle(d) <= 32 << 20 and fake.fake_used(d) == 0
+""")
