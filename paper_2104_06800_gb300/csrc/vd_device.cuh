@@ -183,7 +183,9 @@ __device__ __forceinline__ float vd_ratio_general(const DevParams& P, float r2, 
   const float s = r / alpha;
   const float ls = __log2f(s);
   const float sb = exp2f(P.beta * ls);
-  const float s2b = exp2f((2.0f - P.beta) * ls);
+  // s^(2 - beta); with beta = 2 it is 1 at s = 0 and s = inf too (0 * inf is not)
+  const float lsz = P.beta == 2.0f ? 0.0f : ls;
+  const float s2b = exp2f((2.0f - P.beta) * lsz);
   const float one = 1.0f + sb;
   return P.cgen * alpha * alpha * s2b * one * one;
 }
@@ -219,12 +221,14 @@ __device__ __forceinline__ float vd_l2_general(const DevParams& P, float r2, flo
   const float s = r / alpha;
   const float ls = __log2f(s);
   const float sb = exp2f(P.beta * ls);
-  const float s2b = exp2f((2.0f - P.beta) * ls);
+  // s^(2 - beta); with beta = 2 it is 1 at s = 0 and s = inf too (0 * inf is not)
+  const float lsz = P.beta == 2.0f ? 0.0f : ls;
+  const float s2b = exp2f((2.0f - P.beta) * lsz);
   const float one = 1.0f + sb;
   const float y = P.cgen * alpha * alpha * s2b * one * one;
   if (y < 1e30f) return vd_ell2(y);
   const float l1 = sb < 1e30f ? __log2f(one) : P.beta * ls;   // log2(1 + s^beta)
-  return __log2f(P.cgen * alpha * alpha) + (2.0f - P.beta) * ls + 2.0f * l1;
+  return __log2f(P.cgen * alpha * alpha) + (2.0f - P.beta) * lsz + 2.0f * l1;
 }
 
 __device__ __forceinline__ float vd_l2_beta2(const DevParams& P, float r2) {

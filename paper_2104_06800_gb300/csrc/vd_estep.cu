@@ -78,7 +78,7 @@ k_emission(DevParams P, const float2* __restrict__ posed, const float2* __restri
       const float dx = F.x - vd_em_diff(x, xp);
       const float dy = F.y - vd_em_diff(y, yp);
       const float yv = vd_ratio_y(P, fmaf(dx, dx, dy * dy), fmaf(F.x, F.x, F.y * F.y));
-      l = yv < 1e30f ? __frcp_rn(yv) : 0.0f;   // an overflowing (or 0 * inf) ratio: p1 / P0 = 0
+      l = yv < 1e30f ? __frcp_rn(yv) : 0.0f;   // an overflowing ratio: p1 / P0 = 0
     } else {
       l = obs ? 0.0f : 1.0f;
     }

@@ -516,8 +516,8 @@ struct VdScorePair {
 // and the remainder of the first quotient (Markstein's correction): the bits
 // of a division, but for exact quotients within 2^-23 of a last place of a
 // rounding boundary, in three packed operations.  2 - beta is 0, so the
-// general form's second exponential is 1 (and NaN at log2 s = +-inf, as
-// 0 * inf is).
+// general form's second exponential is 1; at log2 s = +-inf (a zero or infinite
+// residual) the 0 * inf beside it is NaN, which goes to the general form.
 __device__ __forceinline__ void vd_score_scaled(const DevParams& P, vd_f2 r2, vd_f2 nal, vd_f2 ial,
                                                 vd_f2 c, float a0, float a1, float* l0, float* l1) {
   const vd_f2 one = vd_pack(1.0f, 1.0f);
