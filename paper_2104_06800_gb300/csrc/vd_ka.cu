@@ -54,7 +54,8 @@ __device__ __forceinline__ double ka_rcp(double x) {
 // rounded last lies within 2^-51 units in the last place of a / b, so that
 // the result is that of the division unless a / b is that close to a
 // midpoint.  Divisions by one value share its reciprocal: three operations
-// each instead of a division sequence.
+// each instead of a division sequence.  b is normal and below 2^1022: depths and
+// their products are, and the callers see to the Cauchy scale's.
 __device__ __forceinline__ double ka_div(double a, double b, double r) {
   const double q = a * r;
   return fma(fma(-b, q, a), r, q);
@@ -146,7 +147,8 @@ k_ka_accum(const float* __restrict__ theta1, const KaNormal* __restrict__ n1,
   // a NaN is above them: one unsigned compare is 0 <= x <= W - 1
   const unsigned long long xmax = (unsigned long long)__double_as_longlong((double)(c.W - 1));
   const unsigned long long ymax = (unsigned long long)__double_as_longlong((double)(c.H - 1));
-  const double icc = ka_rcp(cc);
+  // (r / c)^2 is 0 for every scale from 2^1000 on, inf among them
+  const double ccq = fmin(cc, 0x1p1000), icc = ka_rcp(ccq);
   const double* sT = Tp.T;
   double acc[NP];
   int n = 0;
@@ -181,12 +183,13 @@ k_ka_accum(const float* __restrict__ theta1, const KaNormal* __restrict__ n1,
     const double DZ = D * Z, iDZ = ka_rcp(DZ), BDZ = ka_div(B, DZ, iDZ);
     const double r = ka_div(A, Z, iZ) - BDZ;
     const double C = conf2 ? (double)conf2[j] : 1.0;
-    const double q = ka_div(r, cc, icc);
+    const double q = ka_div(r, ccq, icc);
     acc[0] += C * (0.5 * cc * cc * log1p(q * q));
     ++n;
     if constexpr (FULL) {
       const double q1 = 1.0 + q * q;
-      const double w = ka_div(C, q1, ka_rcp(q1));
+      // no weight where (r / c)^2 overflows
+      const double w = __double2hiint(q1) == 0x7ff00000 ? 0.0 : ka_div(C, q1, ka_rcp(q1));
       // J = d r / d(omega, v, log s)
       double g3[3] = {ka_div(-m.x, DZ, iDZ), ka_div(-m.y, DZ, iDZ), ka_div(-m.z, DZ, iDZ)};
       const double DZZ = DZ * Z;
