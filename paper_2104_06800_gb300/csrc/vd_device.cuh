@@ -174,6 +174,15 @@ __device__ __forceinline__ vd_f2 vd_sub2(vd_f2 a, vd_f2 b) {
   return r;
 }
 
+// a / b of each half from ib = 1 / b rounded and nb = -b: the first quotient and
+// its remainder (P. Markstein, IBM J. Res. Dev. 34(1), 1990).  The bits of a
+// division, but for exact quotients within 2^-23 of a last place of a rounding
+// boundary, in three packed operations.
+__device__ __forceinline__ vd_f2 vd_div2(vd_f2 a, vd_f2 nb, vd_f2 ib) {
+  const vd_f2 q = vd_mul2(a, ib);
+  return vd_fma2(vd_fma2(q, nb, a), ib, q);
+}
+
 __device__ __forceinline__ float vd_lo(vd_f2 a) { return __uint_as_float((unsigned)a); }
 __device__ __forceinline__ float vd_hi(vd_f2 a) { return __uint_as_float((unsigned)(a >> 32)); }
 

@@ -512,19 +512,16 @@ struct VdScorePair {
   }
 };
 
-// The scaled terms' quotient s = r / alpha comes from the rounded reciprocal
-// and the remainder of the first quotient (Markstein's correction): the bits
-// of a division, but for exact quotients within 2^-23 of a last place of a
-// rounding boundary, in three packed operations.  2 - beta is 0, so the
-// general form's second exponential is 1; at log2 s = +-inf (a zero or infinite
-// residual) the 0 * inf beside it is NaN, which goes to the general form.
+// The scaled terms' quotient s = r / alpha takes the point's reciprocal
+// (vd_div2).  2 - beta is 0, so the general form's second exponential is 1; at
+// log2 s = +-inf (a zero or infinite residual) the 0 * inf beside it is NaN,
+// which goes to the general form.
 __device__ __forceinline__ void vd_score_scaled(const DevParams& P, vd_f2 r2, vd_f2 nal, vd_f2 ial,
                                                 vd_f2 c, float a0, float a1, float* l0, float* l1) {
   const vd_f2 one = vd_pack(1.0f, 1.0f);
   const float ra = vd_lo(r2), rb = vd_hi(r2);
   const vd_f2 r = vd_pack(sqrtf(ra), sqrtf(rb));
-  const vd_f2 q = vd_mul2(r, ial);
-  const vd_f2 s = vd_fma2(vd_fma2(q, nal, r), ial, q);
+  const vd_f2 s = vd_div2(r, nal, ial);
   const vd_f2 ls = vd_pack(__log2f(vd_lo(s)), __log2f(vd_hi(s)));
   const vd_f2 e = vd_add2(ls, ls);
   const vd_f2 u = vd_add2(one, vd_pack(vd_ex2(vd_lo(e)), vd_ex2(vd_hi(e))));
