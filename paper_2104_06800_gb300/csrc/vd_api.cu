@@ -525,7 +525,7 @@ extern "C" vd_status vd_push_flow(vd_ctx* c, int t, const float* uv, long pitch,
 // the launches are the same too and a captured batch stays valid: a batch of
 // RGB-D windows pushes new priors before each run, and captured its graph anew
 // each time (12 windows of 320 x 240 to 1216 x 368, 5 iterations: 39.5 ms a
-// run, 33.2 without the captures).
+// run, 33.2 without the capture, which the first run still makes).
 static void refresh_prior_params(vd_ctx* c) {
   const DevParams before = c->dp;
   const auto version = c->cfg_version;

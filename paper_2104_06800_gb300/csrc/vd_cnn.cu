@@ -672,8 +672,10 @@ __global__ void k_cnn_sum(const double* __restrict__ partial, int n, const int* 
 // reduction this replaced (a float32 chain per thread) 1.9e-7 / 6.6e-8.  On
 // 166 x 72 pixels 8 is above it (1.11e-7 against 1.03e-7) and 4 is not
 // (9.98e-8), so 4.
-// Bound: the issue of the chains and their waits, about 18 us of the 24 (the
-// operand reads of a 640 x 480 layer take 3.5 us, its 39 MB from HBM 5.8).
+// Bound: the latency of a chain's issue, commit and read-back, four chains in
+// flight: the tensor pipe is 15 % busy, DRAM 19 %, the issue slots 32 % (the
+// operand reads of a 640 x 480 layer would take 3.5 us of its 24, its 39 MB from
+// HBM 5.8).
 // With the sum over the blocks 33 us per layer of 32 x 32 channels, 166
 // before (142 and 21; 8 output channels x 9 taps per thread).
 // ---------------------------------------------------------------------------

@@ -169,12 +169,15 @@ __device__ __forceinline__ float vd_slot_candidate(const DevParams& P, uint32_t 
 // lowest slot.  Dropping a candidate whose partial key exceeds a pixel's best
 // key is exact: terms are non-negative, so its full key is at least the
 // partial key, and the best key is that of a finished candidate.
-// Bound: issue slots (71 % busy, the FMA pipe 24 %).  A term's x and y go
-// through packed float32 instructions (vd_f2, one slot for both), FAST leaves
-// the density's other form out of the code, and no term has a branch but the
-// one around its gather: the depth step of a 1216 x 368 window (N = 6, K =
-// 128, with the propagation) 715 -> 617 us, one of 509 x 383 pixels (N = 5, K =
-// 64, stereo prior) 278 -> 238 us, the results the same bits.
+// Bound: with scalar arithmetic issue slots (71 % busy, the FMA pipe 24 %).  A
+// term's x and y now go through packed float32 instructions (vd_f2, one slot
+// for both), FAST leaves the density's other form out of the code, and no term
+// has a branch but the one around its gather: a quarter fewer instructions,
+// the depth step of a 1216 x 368 window (N = 6, K = 128, with the propagation)
+// 715 -> 617 us, one of 509 x 383 pixels (N = 5, K = 64, stereo prior) 278 ->
+// 238 us, the results the same bits.  Now the fixed-latency chain of a term and
+// the ALU pipe's keys, compares and selects (50 %) set the pace, at 61 % of the
+// issue slots.
 // Ring bounds: the pre-pass runs only with fewer than 32 entries in ring 1
 // and adds at most 128; a stage-1 chunk runs only with fewer than 32 entries
 // in ring 2 and adds at most 32.
@@ -431,10 +434,10 @@ VD_UNROLL(VD_KQ_PRE_UNROLL)
 // followed blockDim.x pixels at a time.  Every round settles the first
 // pending pixel of a chain for good, and without a pending pixel every pixel
 // satisfies the definition: the result is exactly the sequential walk.
-// Bound: latency, about 4000 cycles from a pixel's loads to its decision,
-// times the rounds of the slowest chain (19 on a 1216 x 368 window with
-// N = 6, 4.5 on average; a run is 1.2 pixels long on average, the longest
-// 73).  A warp per chain, 38 pixels walked by each lane one after another,
+// Bound: latency.  On a row of a 1216 x 368 window (N = 6) the first decisions
+// take 39 k cycles and a round 5.7 k; a chain needs 4.5 rounds on average, the
+// slowest 17 (a run of one value is 1.3 pixels long on average, the longest
+// 47).  A warp per chain, 38 pixels walked by each lane one after another,
 // took 125 us there and 98 us on 509 x 383 columns with N = 5; this takes 65
 // and 53.
 // ---------------------------------------------------------------------------
@@ -679,10 +682,12 @@ cudaError_t vd_depth_prepare(void) {
 }
 
 // Threads of a block of k_propagate for a chain of L pixels: about ten
-// pixels a thread (measured with 1, 3, 6 and 10 on an earlier form of the
-// kernel: 1216-pixel rows 83, 81, 84 and 72 us, 383-pixel columns 72, 55, 58
-// and 57; more threads a chain leave fewer chains resident, and the later
-// rounds need few).
+// pixels a thread, at least 64 threads.  Whole depth steps beside those with
+// 1, 3 and 6 pixels a thread, each pair timed in turn: 1216-pixel rows 608
+// against 619 us, 627 against 633, 607 against 607; 383-pixel columns 243
+// against 256, 236 against 230, 264 against 264 (64 threads both).  More
+// threads a chain leave fewer chains resident, and the later rounds need few;
+// three pixels a thread gain 3 % on the short columns and lose 1 % on the rows.
 static int prop_threads(int L) {
   return std::min(VD_PROP_MAX_THREADS, std::max(64, (L / 10 + 31) / 32 * 32));
 }

@@ -429,7 +429,7 @@ __device__ __forceinline__ float vd_energy_full(const VdPixel<NF>& px, const Dev
   float xs[NF], ys[NF];
   bool fr[NF];
 #pragma unroll
-  for (int t = 0; t < NF; ++t) {   // projection into frame t + 1 (as vd_flow_term forms it)
+  for (int t = 0; t < NF; ++t) {   // projection into frame t + 1 (as vd_flow_term2 forms it)
     const float* M = sPose + 12 * (t + 1);
     const float hx = fmaf(c, M[9], px.ax[t]);
     const float hy = fmaf(c, M[10], px.ay[t]);

@@ -223,7 +223,10 @@ static inline cudaError_t vd_launch(bool overlap, void (*kern)(K...), dim3 grid,
   return e == cudaSuccess ? cudaGetLastError() : (cudaGetLastError(), e);
 }
 // Whether a context's launches overlap: not those of a batch, whose other
-// windows fill the SMs that a waiting block would hold.
+// windows use the room that a waiting block would hold.  Captured with overlap,
+// batches replayed in 1.15 ms against 1.00 (two windows of 160 x 120), 1.65
+// against 1.20 (four), 6.98 against 6.06 (two of 640 x 480, N = 5) and 32.9
+// against 31.2 (twelve of 320 x 240 to 1216 x 368); one window alone 0.88 both.
 static inline bool vd_overlap(const vd_ctx* c) { return !c->batch_owned; }
 
 // stage profiling hooks (no-ops unless enabled); `n_launch` kernels are counted

@@ -467,8 +467,10 @@ k_p3p_samples(DevParams P, const double* __restrict__ G, const float2* __restric
 // lane L holding the warp's sum of root 32 g + L.  Warp sums are added in
 // fixed order, so the result does not depend on scheduling.
 //
-// Bound: issue slots (31 warp instructions a pixel and root with scalar
-// arithmetic, 21 of them float32).  Two pixels share one packed instruction
+// Bound: with scalar arithmetic issue slots (31 warp instructions a pixel and
+// root, 21 of them float32); now, at 57 % of the slots, the block's final sum,
+// waited for by the warps without a last pass, and the FMA pipe (46 %; a packed
+// instruction holds it for two cycles).  Two pixels share one packed instruction
 // wherever their arithmetic is the same, with the same rounding, and the
 // root's entries lie twice in shared memory for it; the reciprocal and the
 // logarithm skip the rescaling of subnormals that cannot occur.  Same results;
